@@ -99,6 +99,25 @@ __device__ inline bool ans_decode_segment(const uint8_t *states, const uint8_t *
 }
 
 // ---------------------------------------------------------------------------
+// Work units of a block's ANS-coded bitmaps.  A segment of sb bytes keeps
+// W = ceil(sb / 512) lanes busy for at most 512 rounds, so a warp that takes
+// one small bitmap runs as long as one that takes 16 KiB.  Whole segments
+// (16 KiB, 32 lanes) are a unit each; the bitmaps' last, shorter segments
+// share units: their lanes are rounded up to a power of two and laid out by
+// size, largest first, so none crosses a multiple of 32 lanes.
+// ---------------------------------------------------------------------------
+// whole segments of a bitmap, and the lanes (a power of two, 0 for none) of its last one
+__host__ __device__ inline uint32_t ans_full_segs(uint32_t nbytes) { return nbytes / kAnsSeg; }
+__host__ __device__ inline uint32_t ans_tail_lanes(uint32_t nbytes) {
+    const uint32_t sb = nbytes % kAnsSeg;
+    if (!sb) return 0;
+    uint32_t w = ans_seg_lanes(sb), p = 1;
+    while (p < w) p <<= 1;
+    return p;
+}
+__host__ __device__ inline uint32_t ans_units(uint32_t full, uint32_t lanes) { return full + (lanes + 31) / 32; }
+
+// ---------------------------------------------------------------------------
 // Encode one segment (one warp).  src: sb raw bytes (XORed with xr before
 // coding).  The first cap words emitted are staged backwards in stage[0 ..
 // cap) (emission e at cap - 1 - e); later ones go to ovf (global) in

@@ -109,63 +109,81 @@ __device__ inline uint64_t lookback_exclusive_warp(uint64_t *states, int tile, u
     return excl;
 }
 
-// Two chains at once (the same tile in both): lanes 0-15 walk chain A and
-// lanes 16-31 chain B, 16 predecessors per step each; a half that has met
-// its inclusive prefix stops reading while the other goes on.  Called by all
-// 32 lanes; returns both exclusive prefixes in every lane.
-__device__ inline void lookback2_exclusive_warp(uint64_t *states_a, uint64_t *states_b, int tile, uint64_t agg_a,
-                                                uint64_t agg_b, uint64_t &excl_a, uint64_t &excl_b,
-                                                int *timed_out, uint64_t limit_ns) {
-    const int lane = threadIdx.x & 31, half = lane >> 4, hl = lane & 15;
-    uint64_t *states = half ? states_b : states_a;
-    const uint64_t agg = half ? agg_b : agg_a;
-    if (tile == 0) {
-        if (hl == 0) lb_store(&states[0], kLbFlagInc | (agg & kLbValMask));
-        excl_a = excl_b = 0;
-        return;
-    }
-    if (hl == 0) lb_store(&states[tile], kLbFlagAgg | (agg & kLbValMask));
-    uint64_t excl = 0;
+// Two chains walked by a whole CTA (kLbThreads threads): each step reads the
+// states of the kLbThreads predecessors below j at once, so a first wave of
+// CTAs that have all published only their aggregates is crossed in two or
+// three round trips to L2 (a warp's 16 predecessors a step take forty).
+// lb2_publish (one thread) makes the tile's own aggregates visible, before
+// the tile's other work; lookback2_cta waits for the predecessors' (bounded),
+// publishes the inclusive prefixes and returns the exclusive ones in every
+// thread.  Returns true when the wait ran out or a poisoned prefix was met.
+constexpr int kLbThreads = 256;
+constexpr int kLbWarps = kLbThreads / 32;
+__device__ inline void lb2_publish(uint64_t *states_a, uint64_t *states_b, int tile, uint64_t agg_a, uint64_t agg_b) {
+    const uint64_t f = tile == 0 ? kLbFlagInc : kLbFlagAgg;
+    lb_store(&states_a[tile], f | (agg_a & kLbValMask));
+    lb_store(&states_b[tile], f | (agg_b & kLbValMask));
+}
+__device__ inline bool lookback2_cta(uint64_t *states_a, uint64_t *states_b, int tile, uint64_t agg_a, uint64_t agg_b,
+                                     uint64_t &excl_a, uint64_t &excl_b, uint64_t limit_ns, uint32_t (*mins)[4],
+                                     uint64_t (*sums)[2]) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    excl_a = excl_b = 0;
+    if (tile == 0) return false;
     int j = tile - 1;
-    bool done = false;   // (the same in all lanes of a half)
-    bool bad = false;    // an expired wait, or a poisoned prefix met (the same in all lanes)
+    bool bad = false;
     const uint64_t t0 = globaltimer_ns();
     unsigned ns = 32;
     for (;;) {
-        const int k = j - hl;
-        uint64_t v = kLbFlagInc;   // before tile 0: an inclusive zero
-        if (!done && k >= 0) v = lb_load(&states[k]);
-        const uint64_t f = v & (kLbFlagAgg | kLbFlagInc);
-        const uint32_t inc = (__ballot_sync(0xffffffffu, f == kLbFlagInc) >> (16 * half)) & 0xFFFFu;
-        const uint32_t unset = (__ballot_sync(0xffffffffu, f == 0) >> (16 * half)) & 0xFFFFu;
-        const uint32_t pois = (__ballot_sync(0xffffffffu, (v & kLbPoison) != 0) >> (16 * half)) & 0xFFFFu;
-        const uint32_t upto = inc ? ((inc & (0u - inc)) << 1) - 1u : 0xFFFFu;   // lanes up to the nearest one
-        if (__any_sync(0xffffffffu, !done && (unset & upto))) {
-            if (__any_sync(0xffffffffu, globaltimer_ns() - t0 > limit_ns)) {
-                bad = true;
-                break;
-            }
+        const int k = j - t;
+        const uint64_t va = k >= 0 ? lb_load(&states_a[k]) : kLbFlagInc;   // before tile 0: an inclusive zero
+        const uint64_t vb = k >= 0 ? lb_load(&states_b[k]) : kLbFlagInc;
+        const uint64_t fa = va & (kLbFlagAgg | kLbFlagInc), fb = vb & (kLbFlagAgg | kLbFlagInc);
+        // both chains are published one right after the other: a state counts once they agree
+        const bool inc = fa == kLbFlagInc && fb == kLbFlagInc, agg = fa == kLbFlagAgg && fb == kLbFlagAgg;
+        const uint32_t mi = __reduce_min_sync(0xffffffffu, inc ? (uint32_t)t : (uint32_t)kLbThreads);
+        const uint32_t mu = __reduce_min_sync(0xffffffffu, inc || agg ? (uint32_t)kLbThreads : (uint32_t)t);
+        // (one thread's clock decides for the CTA)
+        if (lane == 0) {
+            mins[warp][0] = mi;
+            mins[warp][1] = mu;
+            mins[warp][2] = t == 0 && globaltimer_ns() - t0 > limit_ns;
+        }
+        __syncthreads();
+        uint32_t ti = kLbThreads, tu = kLbThreads;
+#pragma unroll
+        for (int w = 0; w < kLbWarps; w++) { ti = min(ti, mins[w][0]); tu = min(tu, mins[w][1]); }
+        const bool expired = mins[0][2] != 0;
+        const bool take = (uint32_t)t <= ti;   // up to the nearest inclusive prefix
+        uint64_t xa = take ? va & kLbValMask : 0ull, xb = take ? vb & kLbValMask : 0ull;
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            xa += __shfl_xor_sync(0xffffffffu, xa, o);
+            xb += __shfl_xor_sync(0xffffffffu, xb, o);
+        }
+        const bool pois = (uint32_t)t == ti && ((va | vb) & kLbPoison) != 0;
+        if (lane == 0) { sums[warp][0] = xa; sums[warp][1] = xb; }
+        const bool anyp = __syncthreads_or(pois) != 0;
+        if (tu < ti) {   // a state needed is not there yet
+            if (expired) { bad = true; break; }
             __nanosleep(ns);
-            if (ns < 1024) ns <<= 1;
+            if (ns < 512) ns <<= 1;
+            __syncthreads();
             continue;
         }
-        uint64_t x = (!done && ((upto >> hl) & 1u)) ? (v & kLbValMask) : 0ull;
 #pragma unroll
-        for (int o = 8; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);   // within the half
-        if (__any_sync(0xffffffffu, !done && (pois & inc & (0u - inc)) != 0)) bad = true;
-        if (!done) {
-            excl += x;
-            if (inc) done = true;
-            else j -= 16;
-        }
-        if (__all_sync(0xffffffffu, done)) break;
+        for (int w = 0; w < kLbWarps; w++) { excl_a += sums[w][0]; excl_b += sums[w][1]; }
+        if (ti < (uint32_t)kLbThreads) { bad = anyp; break; }
+        j -= kLbThreads;
+        __syncthreads();
     }
-    // a poisoned or partial prefix in either chain makes both chains' prefixes
-    // unusable downstream (the block's offsets come from both)
-    if (bad) *timed_out = 1;
-    if (hl == 0) lb_store(&states[tile], kLbFlagInc | (bad ? kLbPoison : 0ull) | ((excl + agg) & kLbValMask));
-    excl_a = __shfl_sync(0xffffffffu, excl, 0);
-    excl_b = __shfl_sync(0xffffffffu, excl, 16);
+    __syncthreads();
+    if (t == 0) {
+        const uint64_t p = bad ? kLbPoison : 0ull;
+        lb_store(&states_a[tile], kLbFlagInc | p | ((excl_a + agg_a) & kLbValMask));
+        lb_store(&states_b[tile], kLbFlagInc | p | ((excl_b + agg_b) & kLbValMask));
+    }
+    return bad;
 }
 
 }  // namespace pv

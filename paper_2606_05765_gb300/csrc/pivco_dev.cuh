@@ -566,7 +566,7 @@ cudaError_t launch_decode_merge(const uint8_t *comp, const uint64_t *comp_off, i
                                 const uint64_t *out_off, uint8_t *ws, size_t ws_bytes, int32_t *status,
                                 cudaStream_t st);
 cudaError_t launch_decode_dir(const uint8_t *comp, const uint64_t *comp_off, int nblk, uint8_t *ws, size_t ws_bytes,
-                              int32_t *status, cudaStream_t st);
+                              int32_t *status, cudaStream_t st, bool access);
 cudaError_t launch_golomb_plan(const uint8_t *in, const uint64_t *blk_off, int nblk, uint64_t *rec_size,
                                int32_t *status, cudaStream_t st);
 cudaError_t launch_golomb_encode(const uint8_t *in, const uint64_t *blk_off, int nblk, uint8_t *out,
