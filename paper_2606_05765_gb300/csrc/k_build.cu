@@ -540,13 +540,32 @@ __device__ inline void build_layout_block(int b, const uint32_t *h, const uint8_
                     const uint64_t n1 = c >= 0 ? L.nv[c] : h[-c - 1];
                     L.sel[t] = ans_select(L.nv[t], n1, L.depth[t], sp);
                 }
-                // a big block: some level (depth >= 1) of the whole block
-                // does not fit an encoder level buffer (spans of whole
-                // 16-byte units), so the chunked encoder splits it
+                // a big block is coded chunk by chunk by several CTAs: some
+                // level (depth >= 1) of the whole block does not fit an
+                // encoder level buffer (spans of whole 16-byte units), or
+                // the batch has too few blocks to fill the chip with one CTA
+                // each
+                if (t == 0 && gridDim.x <= kEncFewBlocks && n >= kEncFewSize && maxd > 1) L.big = 1;
+                unsigned long long part = n;
                 if (t >= 1 && t < maxd) {
-                    uint64_t lvl = 0;
-                    for (int v = fst[t]; v < fst[t + 1]; v++) lvl += ((uint64_t)L.nv[v] + 7u) & ~7ull;
+                    uint64_t lvl = 0, raw = 0;
+                    for (int v = fst[t]; v < fst[t + 1]; v++) {
+                        lvl += ((uint64_t)L.nv[v] + 15u) & ~15ull;
+                        raw += L.nv[v];
+                    }
                     if (lvl > (uint64_t)kEBuf && enc_nchunks(n) >= 2) L.big = 1;
+                    // a part's level: its share of the level and the spans' rounding, 10 % to spare
+                    const uint64_t room = (uint64_t)kEBuf - 16ull * (uint32_t)(fst[t + 1] - fst[t]);
+                    if (raw) part = room * n / raw / 10 * 9;
+                }
+                if (t < 32) {
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) {
+                        const unsigned long long y = __shfl_xor_sync(0xffffffffu, part, o);
+                        part = y < part ? y : part;
+                    }
+                    // (in whole rounds of the encoder's eight windows, where it holds one)
+                    if (t == 0) L.part = (uint32_t)(part >= 8192 ? part & ~8191ull : part & ~1023ull);
                 }
                 __syncthreads();
             if (t < 32) {

@@ -28,6 +28,7 @@
 //              decoded in shorter chunks whose bit ranges are found top-down
 //              from popcounts.
 #include "ans_dev.cuh"
+#include "levels.cuh"
 #include "lookback.cuh"
 
 namespace pv {
@@ -53,16 +54,6 @@ __device__ inline uint32_t dec_dir_bits(const uint8_t *ws) { return reinterpret_
 __device__ inline bool dec_all_dirs(const uint8_t *ws) { return (reinterpret_cast<const uint32_t *>(ws)[7] >> 31) != 0; }
 
 __host__ __device__ inline uint32_t scratch_stride(uint32_t raw) { return ((raw + 15u) & ~15u) + 16u; }
-
-__device__ inline uint32_t warp_inclusive(uint32_t x) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    return x;
-}
 
 // The dynamic shared memory of every kernel here: the merge's selector table
 // (1 KiB), then what the item at hand needs.  The big steps are functions of
@@ -1323,9 +1314,7 @@ cudaError_t launch_ans_decode_planned(const uint8_t *comp, const uint64_t *comp_
 // 20-300 KB, 60-120 symbols, canonical tree: 377 us before, 220 us now.
 // ---------------------------------------------------------------------------
 constexpr int kTileWarps = kDecWarps;
-constexpr int kWinMax = 512;                   // windows of all levels below the root
-constexpr uint32_t kGrp = 32;                  // symbols of a group (one lane's bitmap word)
-constexpr uint32_t kWin = 32 * kGrp;           // symbols of a full window
+static_assert(kTileWarps == kLvlWarps, "the level tables are laid out by all warps");
 constexpr int kStripMax = 256;                 // strips of root windows (a window each up to 2^18 symbols)
 
 struct TileSrc {
@@ -1345,6 +1334,7 @@ struct TileJob {
 };
 
 struct __align__(16) CtaTile {
+    static constexpr int kBuf = kLvlBuf;
     uint8_t buf[2][kLvlBuf + kWSlack];         // level buffers: depth d writes buf[d & 1]
     uint32_t pos[256];                         // bit address of node v's next bit (bit 31: in the ANS scratch)
     uint32_t dem[256];                         // bits of node v in the current chunk
@@ -1565,102 +1555,6 @@ __device__ inline void put_step(uint8_t *dst, int s, uint2 o, uint32_t nb, uint3
     if (s == 3 && lane == 31 && nb + mis > 1024) st_bytes(dst + 1016, cur, 8 - (int)mis, (int)nb - 1016);
 }
 
-// Spans, groups and windows of every level for the current demands, by the
-// whole CTA: warp w lays out levels w, w + 8, ... (a level's spans, groups
-// and flat windows are one packed scan over its own nodes); the levels'
-// window tables then follow one another in depth order.  Spans start on
-// 16-byte boundaries, so a lane stores its 32 symbols in two vectors (eight
-// 4-byte stores 32 bytes apart were 64 wavefronts a window).  False (in
-// every thread) when a level (depth >= 1) does not fit a buffer or the
-// windows do not fit their table.
-__device__ inline bool ct_layout(CtaTile &S) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int maxd = S.maxd;
-    bool fits = true;
-    for (int d = warp; d < maxd; d += kTileWarps) {
-        if (d == 0) continue;   // the root has no span; its windows are strips
-        const int f0 = S.first[d], f1 = S.first[d + 1];
-        // bytes << 40 | groups of ordinary nodes << 20 | flat windows << 10 | ordinary nodes
-        uint64_t carry = 0;
-        for (int base = f0; base < f1; base += 32) {
-            const int v = base + lane;
-            uint64_t x = 0;
-            bool flat = false;
-            uint32_t dv = 0;
-            if (v < f1) {
-                dv = S.dem[v];
-                flat = ch_flat_d(S.ch[v]) != 0;
-                if (dv > (uint32_t)kLvlBuf) { fits = false; dv = kLvlBuf; }
-                const uint32_t by = (dv + 15u) & ~15u;
-                x = ((uint64_t)by << 40) |
-                    (flat ? (uint64_t)((dv + kWin - 1) / kWin) << 10 : ((uint64_t)max(1u, (dv + kGrp - 1) / kGrp) << 20) | 1u);
-            }
-            uint64_t inc = x;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) inc += y;
-            }
-            const uint64_t ex = carry + inc - x;
-            if (v < f1) {
-                S.sp[v] = (uint16_t)min((uint64_t)kLvlBuf, ex >> 40);
-                if (flat) {
-                    S.fw[v] = (uint16_t)((ex >> 10) & 1023u);
-                } else {
-                    const uint32_t i = (uint32_t)f0 + ((uint32_t)ex & 1023u);
-                    S.onode[i] = (uint8_t)v;
-                    S.gs[i] = (uint16_t)((ex >> 20) & 0xFFFFFu);
-                }
-            }
-            carry += __shfl_sync(0xffffffffu, inc, 31);
-        }
-        if ((carry >> 40) > (uint64_t)kLvlBuf) fits = false;
-        const uint32_t G = (uint32_t)(carry >> 20) & 0xFFFFFu, nwo = (G + 31) >> 5;
-        if (G > 0xFFFFu) fits = false;
-        if (lane == 0) {
-            S.lg[d] = (uint16_t)G;
-            S.no[d] = (uint16_t)(carry & 1023u);
-            S.nwo[d] = (uint16_t)nwo;
-            S.nw[d] = (uint16_t)(nwo + ((uint32_t)(carry >> 10) & 1023u));
-        }
-    }
-    __syncthreads();
-    // window table offsets: lane d holds level d's windows (none at the root)
-    const uint32_t nwin_l = lane >= 1 && lane < maxd ? (uint32_t)S.nw[lane] : 0u;
-    uint32_t wi = nwin_l;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
-        if (lane >= o) wi += y;
-    }
-    if (__shfl_sync(0xffffffffu, wi, 31) > (uint32_t)kWinMax) fits = false;
-    const uint32_t wn_l = wi - nwin_l;
-    for (int d = warp; d < maxd; d += kTileWarps) {
-        const uint32_t wn = __shfl_sync(0xffffffffu, wn_l, d);
-        if (d == 0) continue;
-        if (lane == 0) S.wn_off[d] = (uint16_t)min(wn, (uint32_t)kWinMax);
-        // ordinary windows: the last ordinary node whose first group is at or before the window's first
-        const uint32_t nwo = S.nwo[d], no = S.no[d];
-        const int f0 = S.first[d], f1 = S.first[d + 1];
-        for (uint32_t i = lane; i < nwo && wn + i < (uint32_t)kWinMax; i += 32) {
-            int lo = 0, hi = (int)no;
-            while (hi - lo > 1) {
-                const int m = (lo + hi) >> 1;
-                if ((uint32_t)S.gs[f0 + m] <= 32u * i) lo = m; else hi = m;
-            }
-            S.wnode[wn + i] = (uint8_t)lo;
-        }
-        // flat windows: their node
-        if (no != (uint32_t)(f1 - f0))
-            for (int v = f0 + lane; v < f1; v += 32)
-                if (ch_flat_d(S.ch[v])) {
-                    const uint32_t w0 = wn + nwo + S.fw[v], nf = (min(S.dem[v], (uint32_t)kLvlBuf) + kWin - 1) / kWin;
-                    for (uint32_t i = 0; i < nf && w0 + i < (uint32_t)kWinMax; i++) S.wnode[w0 + i] = (uint8_t)v;
-                }
-    }
-    return !__syncthreads_or(!fits);
-}
-
 // Demands of a chunk of C root symbols from the current cursors, top-down:
 // a node's popcount over its range splits its demand between its children
 // (one warp).
@@ -1829,20 +1723,8 @@ __device__ __forceinline__ bool ct_level(CtaTile &S, const TileSrc &src, int d, 
         const uint32_t i = base + warp;
         uint32_t v = 0, q = 0, w = 0, inc = 0, left = 0;   // left: symbols of the node from this group on (0: none)
         if (i < nwo) {
-            const uint32_t g = 32u * i + lane, u = S.wnode[wn + i];
-            // the nodes after u that start in the window (every node has a group)
-            const uint32_t cand = u + 1 + lane;
-            uint32_t bit = 0;
-            if (cand < S.no[d]) {
-                const uint32_t s = (uint32_t)S.gs[f0 + cand] - 32u * i;
-                if (s < 32) bit = 1u << s;
-            }
-            const uint32_t idx = f0 + u + __popc(__reduce_or_sync(0xffffffffu, bit) & (0xFFFFFFFFu >> (31 - lane)));
-            v = S.onode[idx];
-            q = g - S.gs[idx];
-            const uint32_t dv = S.dem[v];
-            if (g < S.lg[d] && kGrp * q < dv) {
-                left = dv - kGrp * q;
+            left = lvl_locate(S, d, wn, f0, i, v, q);
+            if (left) {
                 w = tile_bits(src, S.pos[v], kGrp * q);
                 if (left < 32) w &= (1u << left) - 1u;
             }
@@ -1942,7 +1824,7 @@ __device__ __forceinline__ int ct_decode() {
             if (warp == 0) ct_demand(S, src, V, C);
             __syncthreads();
         }
-        if (!ct_layout(S)) {
+        if (!lvl_layout(S)) {
             chunked = true;
             C = max(32u, (C / 2) & ~31u);
             continue;

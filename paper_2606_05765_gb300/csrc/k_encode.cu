@@ -1,80 +1,74 @@
 // Encode kernel: per-node bitmap emission by stable partition (Sec. 4, Sec. 2.4.1).
 //
 // One CTA encodes one block, top-down, level by level; its warps share two
-// level buffers.  The block is coded in chunks whose levels fit those
-// buffers (usually a few of the planning pass's chunks, whose histograms
-// give every node's symbol count in the chunk; a chunk too large for the
-// buffers is cut and counted again).  A node's bitmap holds, in block order,
-// the code bit of every symbol passing through it, so the chunk's bits of
-// node v start at the symbols under v in the chunks before it: the cursors
-// advance by each chunk's counts.  Per level, the symbols of every node are
-// cut into groups of 32 (one lane each) and windows of 32 groups, which the
-// warps take in rounds of eight.  A lane's 32 code bits at the node's depth
-// form one bitmap word (written to the record at the node's cursor; words
-// shared with a neighbour are ORed into the zeroed body), and its symbols
-// are stably partitioned into the internal children's spans (EPF / EPL /
-// EPR / EPN of Sec. 2.4.1) at the zeros / ones of the node before the group:
-// a segmented warp scan within the window, the windows' summaries across a
-// round (one barrier), a carry across rounds.  Below the root a symbol
-// travels as its remaining code bits, most significant first in 16 bits, so
-// a node's bit is bit 15 and the child receives the value shifted left by
-// one.  A flat node (Sec. 2.2.3) takes the top D bits of each value, its
-// symbol's index in the flat group, and packs them D bits per symbol.
+// level buffers.  A block whose levels fit them is coded in one part (the
+// planning pass's chunk histograms give every node's symbol count); a big
+// block is coded in parts of a length the plan has chosen, by several CTAs
+// (one planning chunk, or a share of one, each), a part's counts taken from
+// the input.  A node's bitmap holds, in block order, the code bit of every
+// symbol passing through it, so a part's bits of node v start at the symbols
+// under v in the parts before it: the cursors advance by each part's counts.
+//
+// Below the root a symbol travels as its code index, its place in the order
+// of codes, in one byte: the leaves under a node are consecutive there, so
+// its code bit at node v is (index >= split of v), one byte compare, and the
+// index in a flat node's group (Sec. 2.2.3) a subtraction.  Per level, the
+// symbols of every node are cut into groups of 32 (one bitmap word) and
+// windows of 32 groups, which the warps take in rounds of eight.  In a window
+// a lane takes 8 consecutive symbols at a time, so that neighbouring lanes
+// read and write neighbouring bytes: the compare gives the lane a byte of the
+// bitmap, the window's 128 bytes become one word per lane (written to the
+// record at the node's cursor; words shared with a neighbour are ORed into
+// the zeroed body), and the symbols are stably partitioned into the internal
+// children's spans (EPF / EPL / EPR / EPN of Sec. 2.4.1) at the zeros / ones of
+// the node before the group: a warp scan within the window, the windows'
+// counts across a round (one barrier), a carry across rounds.
+//
+// What bounds it: instruction issue and shared-memory wavefronts.  (With 32
+// symbols of 16 bits to a lane, a window took about 800 instructions and 200
+// wavefronts.)  MEAS_ENC
 
-#include "pivco_dev.cuh"
+#include "levels.cuh"
 
 namespace pv {
 
 constexpr int kEncThreads = 256;
 constexpr int kEncWarps = kEncThreads / 32;
-constexpr int kEncCtasPerSm = 3;
-constexpr int kESlack = 48;                 // over-read room (symbols)
-constexpr int kEWinPerLvl = 32;             // windows of a level below the root (<= kEBuf/32 + 128 groups)
+constexpr int kEncCtasPerSm = 4;
+static_assert(kEncWarps == kLvlWarps, "the level tables are laid out by all warps");
 
-struct EncWin {                             // one window of a round
-    uint32_t sum;                           // ones of its last node from that node's start in the window
-    uint32_t flags;                         // 1 its first node starts at its first group, 2 a node starts in it, 4 active
-};
-
-template <int kBufT, int kWinT>
-struct __align__(16) EncSmemT {
-    static constexpr int kBuf = kBufT;      // symbols per level buffer
-    static constexpr int kWin = kWinT;      // windows of a level below the root (>= (kBuf / 32 + 256) / 32)
-    uint16_t buf[2][kBufT + kESlack];       // depth d >= 1 reads buf[d & 1], writes its children to the other
-                                            // (spans start on 16-byte boundaries)
-    uint32_t pos[256];                      // bit address of node v's first bit of the current chunk
-    uint32_t dem[256];                      // symbols of node v in the current chunk
+struct __align__(16) EncSmem {
+    static constexpr int kBuf = kEBuf;      // symbols per level buffer
+    uint8_t buf[2][kEBuf + 16];             // depth d >= 1 reads buf[d & 1], writes its children to the other
+    uint32_t pos[256];                      // bit address of node v's first bit of the current part
+    uint32_t dem[256];                      // symbols of node v in the current part
     uint32_t ch[256];                       // children word (node-table format; ch_flat for a flat node)
-    uint32_t bitsrc[256];                   // bit address of node v's bitmap in the record
-    uint32_t nv[256];                       // bits of node v's body (n_v, n_v D for a flat node)
-    uint16_t code16[256];                   // code of symbol s, most significant bit at bit 15 (0: absent)
-    uint16_t sp[256];                       // first symbol of node v's span in its level buffer
-    uint16_t gs[256];                       // first 32-symbol group of node v within its level
-    uint16_t lg[16];                        // groups of each level
-    uint8_t wnode[16][kWinT];               // node holding the first group of each window of a level
-    EncWin win[2][kEncWarps];               // window summaries, two rounds deep
-    uint8_t ci[256];                        // canonical index of symbol s (its place in (length, symbol) order)
-    uint8_t nlo[256];                       // node v's leaves are canonical indices nlo[v] .. nhi1[v]
+    uint32_t end[256];                      // bit address of the end of node v's body (of the item's part of it)
+    uint32_t strip[kEncWarps][72];          // a window's bitmap bytes, or a flat step's packed indices
+    uint32_t wtot[2][kEncWarps];            // ones of a round's ordinary windows, two rounds deep
+    uint16_t sp[256], gs[256], fw[256];     // (levels.cuh; fw of an ordinary node: ones before its first group in
+                                            // that group's window)
+    uint16_t wpre[kWinMax];                 // prefixes of earlier rounds (levels of more than 8 windows)
+    uint16_t lg[16], no[16], nwo[16], nw[16], wn_off[16];
+    uint8_t onode[256];
+    uint8_t wnode[kWinMax];
+    uint8_t split[256];                     // first code index of node v's right child; a flat node's first index
+    uint8_t ci[256];                        // code index of symbol s; 255 for a symbol without a code
+    uint8_t nlo[256];                       // node v's leaves are code indices nlo[v] .. nhi1[v]
     uint8_t nhi1[256];
+    uint32_t lut[256];                      // byte selectors that bring the symbols of a bitmap byte's zeros to the
+                                            // front (first four in the low half)
     uint32_t pmask[8];                      // symbols that have a code
     uint32_t hot;                           // the symbol with the shortest code (the most frequent one)
-    uint32_t bad, fits;
-    uint32_t lvl_max;                       // symbols of the largest level below the root (a try's layout)
+    uint32_t bad, lvl_max;                  // symbols of the largest level below the root (a part that did not fit)
     uint8_t first[17];
     uint8_t maxd;
     uint8_t pad[14];
 };
-// the whole-block encoder's buffers (3 CTAs per SM), and the chunk
-// encoder's (2 CTAs per SM, parts of big blocks almost twice as long)
-using EncSmem = EncSmemT<kEBuf, kEWinPerLvl>;
-constexpr int kEBufBig = 25600;
-constexpr int kEncChunkCtasPerSm = 2;
-using EncSmemBig = EncSmemT<kEBufBig, 36>;
+static_assert(kEncCtasPerSm * (sizeof(EncSmem) + 64 + 1024) <= 228 * 1024, "encoder CTAs per SM");
 static_assert(offsetof(BlockLayout, ci) <= sizeof(EncSmem::buf[1]) && offsetof(BlockLayout, ci) % 16 == 0,
               "the staged part of the layout fits a level buffer");
 static_assert(sizeof(EncSmem::buf[0]) >= 4 * (288 + 256 + 257), "a level buffer holds the counting scratch");
-static_assert(kEncChunkCtasPerSm * (sizeof(EncSmemBig) + 1024) <= 228 * 1024, "chunk encoder CTAs per SM");
-static_assert((kEBufBig / 32 + 256) / 32 <= 36, "window table of the chunk encoder");
 
 template <typename F, typename G>
 __device__ inline uint32_t warp_scan_loop(int n, F f, G out) {
@@ -151,8 +145,7 @@ __device__ inline void hist_fold_hot(uint32_t *hist, uint32_t h) {
 // leaves under a node are the contiguous canonical range nlo .. nhi1, so its
 // count is a difference of two prefix sums.  One warp; hc (256) and ps (257)
 // are scratch.
-template <typename SM>
-__device__ inline void enc_counts(const SM &S, const uint32_t *h, uint32_t *cnt, uint32_t *hc, uint32_t *ps) {
+__device__ inline void enc_counts(const EncSmem &S, const uint32_t *h, uint32_t *cnt, uint32_t *hc, uint32_t *ps) {
     const int lane = threadIdx.x & 31;
     const int V = S.first[S.maxd];
 #pragma unroll
@@ -179,87 +172,6 @@ __device__ inline void enc_counts(const SM &S, const uint32_t *h, uint32_t *cnt,
     __syncwarp();
 }
 
-// Spans, groups and window nodes of level d for the current demands (one
-// warp; the levels are independent).  False when the level (depth >= 1)
-// does not fit a buffer or has more windows than its window-node table.
-template <typename SM>
-__device__ inline bool enc_layout_level(SM &S, int d) {
-    constexpr int kBuf = SM::kBuf;
-    const int lane = threadIdx.x & 31;
-    bool fits = true;
-    const int f0 = S.first[d], f1 = S.first[d + 1];
-    uint64_t carry = 0;
-    uint32_t raw = 0;   // this lane's nodes' symbols, rounded as spans are (capped: only sizes near a buffer matter)
-    for (int base = f0; base < f1; base += 32) {
-        const int v = base + lane;
-        uint64_t x = 0;
-        if (v < f1) {
-            const uint32_t dv = S.dem[v];
-            raw = min(raw + ((min(dv, 1u << 24) + 7u) & ~7u), 1u << 25);
-            if (d && dv > (uint32_t)kBuf) fits = false;
-            const uint32_t el = d ? ((min(dv, (uint32_t)kBuf) + 7u) & ~7u) : 0u;   // spans of whole 16-byte units
-            x = ((uint64_t)el << 32) | max(1u, (dv + 31u) >> 5);
-        }
-        uint64_t inc = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        const uint64_t ex = carry + inc - x;
-        if (v < f1) {
-            S.sp[v] = (uint16_t)min((uint64_t)kBuf, ex >> 32);
-            S.gs[v] = (uint16_t)ex;
-        }
-        carry += __shfl_sync(0xffffffffu, inc, 31);
-    }
-    if (d && (carry >> 32) > (uint64_t)kBuf) fits = false;
-    if ((uint32_t)carry > 0xFFFFu) fits = false;
-    const uint32_t G = (uint32_t)carry & 0xFFFFu;
-    const uint32_t lraw = __reduce_add_sync(0xffffffffu, raw);
-    if (lane == 0) {
-        S.lg[d] = (uint16_t)G;
-        if (d) atomicMax(&S.lvl_max, lraw);
-    }
-    __syncwarp();
-    if (d) {
-        const uint32_t nwin = (G + 31) >> 5;
-        if (nwin > (uint32_t)SM::kWin) fits = false;
-        for (uint32_t i = lane; i < nwin && i < (uint32_t)SM::kWin; i += 32) {
-            int lo = f0, hi = f1;
-            while (hi - lo > 1) {
-                const int m = (lo + hi) >> 1;
-                if ((uint32_t)S.gs[m] <= 32u * i) lo = m; else hi = m;
-            }
-            S.wnode[d][i] = (uint8_t)lo;
-        }
-    }
-    __syncwarp();
-    return __all_sync(0xffffffffu, fits);
-}
-
-// The carry into this warp's window of the round (the ones, before the
-// window, of the node that runs into it) and the carry into the next round;
-// every warp calls it after the round's summaries are written.
-template <typename SM>
-__device__ inline uint32_t enc_round_carry(const SM &S, uint32_t par, uint32_t &rc_sum) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const EncWin x = lane < kEncWarps ? S.win[par][lane] : EncWin{0u, 0u};
-    uint32_t val = x.sum, seg = (x.flags >> 1) & 1u;
-#pragma unroll
-    for (int o = 1; o < kEncWarps; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, val, o), f = __shfl_up_sync(0xffffffffu, seg, o);
-        if (lane >= o && !seg) { val += y; seg |= f; }
-    }
-    if (!seg) val += rc_sum;
-    const uint32_t prev = __shfl_up_sync(0xffffffffu, val, 1);
-    const uint32_t c = (x.flags & 1u) ? 0u : (lane ? prev : rc_sum);
-    const uint32_t cin = __shfl_sync(0xffffffffu, c, warp);
-    const uint32_t act = __ballot_sync(0xffffffffu, (x.flags & 4u) != 0);   // window 0 always is
-    rc_sum = __shfl_sync(0xffffffffu, val, 31 - __clz(act));
-    return cin;
-}
-
 // Writes bits bw (vl of them valid) of one node at bit address a of the
 // record.  Lanes of the same node hold consecutive 32-bit runs; a lane
 // stores the aligned word its run starts in, completed with the previous
@@ -282,126 +194,435 @@ __device__ inline void enc_put_bits(uint32_t *rec32, bool act, uint32_t v, uint3
     if (hi && !next_same) atomicOr(&rec32[wi + 1], hi);
 }
 
-// The top bit of each of the 8 16-bit values in x0..x3 (value j at bits j)
-__device__ inline uint32_t top_bits8(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3) {
-    const uint32_t h0 = __byte_perm(x0, x1, 0x7531), h1 = __byte_perm(x2, x3, 0x7531);
-    const uint32_t b0 = ((h0 & 0x80808080u) * 0x00204081u) >> 28;
-    const uint32_t b1 = ((h1 & 0x80808080u) * 0x00204081u) >> 28;
-    return b0 | (b1 << 4);
+// ---- bytes ----
+// bit j: whether byte j of the 8 in x0, x1 is marked in bit 7 of m0, m1 (the
+// dot product weighs bits 3 and 7 of byte j by 2^j)
+__device__ inline uint32_t gather8(uint32_t m0, uint32_t m1) {
+    return __dp4a(((m0 >> 4) & 0x08080808u) | (m1 & 0x80808080u), 0x08040201u, 0u) >> 3;
 }
+// bytes of x not below those of s, marked in bit 7
+__device__ inline uint32_t ge4(uint32_t x, uint32_t s) {
+    const uint32_t t = (x | 0x80808080u) - (s & 0x7F7F7F7Fu);
+    return (x & ~s) | (~(x ^ s) & t);
+}
+// bytes of x that are zero, marked in bit 7
+__device__ inline uint32_t eq4(uint32_t x) { return ~(((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x); }
+// the first n bytes (0..4) of a word
+__device__ inline uint32_t mask4(int n) { return n >= 4 ? 0xFFFFFFFFu : (n <= 0 ? 0u : (1u << (8 * n)) - 1u); }
 
 __device__ inline uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ inline void sts16(uint32_t a, uint32_t v) {
-    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
+template <int K>
+__device__ inline void sts8(uint32_t a, uint32_t v) {
+    asm volatile("st.shared.u8 [%0+%2], %1;" ::"r"(a), "r"(v), "n"(K) : "memory");
 }
 
-// Stable partition of up to 32 symbols (values y[j], bits in bw, vl valid)
-// into the left (bit 0) and right (bit 1) spans of the next level, given as
-// shared-memory byte addresses.  Only internal children keep symbols: with
-// both internal every symbol is stored (one address select each); with one,
-// only that side's symbols are.
-__device__ inline void enc_split(uint32_t la, uint32_t ra, bool i0, bool i1, const uint32_t (&y)[16], uint32_t bw,
-                                 uint32_t vl) {
-    const uint32_t vm = vl >= 32 ? 0xFFFFFFFFu : ((1u << vl) - 1u);
-    if (i0 && i1) {
-        // the j-th symbol goes to ra + 2 ones_before(j) or la + 2 (j - ones_before(j))
-        uint32_t ob = 0;
-        if (vl >= 32) {
+// 8 input bytes at p, `mis` bytes past a 4-byte boundary (bytes at or past
+// `end` are not read; at least one byte is before it)
+__device__ inline uint2 ldg8(const uint8_t *p, uint32_t mis, const uint8_t *end) {
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(p - mis);
+    const uint8_t *q = p - mis;
+    if (mis == 0) {
+        if (!(reinterpret_cast<uintptr_t>(p) & 7) && p + 8 <= end) return __ldg(reinterpret_cast<const uint2 *>(p));
+        return make_uint2(__ldg(w), q + 4 < end ? __ldg(w + 1) : 0u);
+    }
+    const uint32_t a = __ldg(w), b = q + 4 < end ? __ldg(w + 1) : 0u, c = q + 8 < end ? __ldg(w + 2) : 0u;
+    return make_uint2(__funnelshift_r(a, b, 8 * mis), __funnelshift_r(b, c, 8 * mis));
+}
+
+// What a window's groups carry to their lanes' steps: the bitmap word, the
+// children's next places in the level below (of the group's first symbol,
+// left | right << 16) and bits 0..5 its symbols, 6 / 7: internal left / right
+// child.
+struct EncGrp {
+    uint32_t w, a, b;
+};
+
+// Partitions a window: y[2 s], y[2 s + 1] are the lane's 8 symbols of step s.
+// A byte permute by the bitmap byte brings the symbols of its zeros to the
+// front; the k-th then goes to the k-th place of the left span or, past the
+// zeros, of the right one.
+__device__ inline void enc_partition(const EncSmem &S, uint32_t base, const EncGrp &G, const uint32_t (&y)[8]) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t sub = lane & 3, below = (1u << (8 * sub)) - 1u;
+    const bool two = __all_sync(0xffffffffu, (G.b & 0xFFu) == (32u | 0xC0u));   // full groups, both children internal
+    if (!__any_sync(0xffffffffu, (G.b & 0xC0u) != 0)) return;
 #pragma unroll
-            for (int j = 0; j < 32; j++) {
-                const uint32_t bit = (bw >> j) & 1u;
-                const uint32_t val = (y[j >> 1] >> (16 * (j & 1))) << 1;
-                sts16(bit ? ra + ob : la + (2u * j - ob), val);
-                ob += 2u * bit;
-            }
+    for (int s = 0; s < 4; s++) {
+        const int own = 8 * s + (lane >> 2);
+        const uint32_t ws = __shfl_sync(0xffffffffu, G.w, own), as = __shfl_sync(0xffffffffu, G.a, own);
+        const uint32_t r = __popc(ws & below);
+        const uint32_t la = base + (as & 0xFFFFu) + 8 * sub - r;
+        uint32_t b8 = (ws >> (8 * sub)) & 0xFFu;
+        uint32_t st = 0xFFu;   // sorted symbols stored
+        if (!two) {
+            const uint32_t bs = __shfl_sync(0xffffffffu, G.b, own);
+            const int nv = max(0, min(8, (int)(bs & 63u) - 8 * (int)sub));   // valid symbols of the lane's 8
+            b8 |= (0xFFu << nv) & 0xFFu;                                      // (the others sort behind the ones)
+            const uint32_t zm = (1u << (8u - __popc(b8))) - 1u;              // the zeros
+            st = (bs & 0x40u ? zm : 0u) | (bs & 0x80u ? ((1u << nv) - 1u) & ~zm : 0u);
+        }
+        const uint32_t z = 8u - __popc(b8), e = S.lut[b8], rb = base + (as >> 16) + r - z;
+        const uint32_t s0 = __byte_perm(y[2 * s], y[2 * s + 1], e), s1 = __byte_perm(y[2 * s], y[2 * s + 1], e >> 16);
+        if (two) {
+            sts8<0>(z > 0 ? la : rb, s0);
+            sts8<1>(z > 1 ? la : rb, s0 >> 8);
+            sts8<2>(z > 2 ? la : rb, s0 >> 16);
+            sts8<3>(z > 3 ? la : rb, s0 >> 24);
+            sts8<4>(z > 4 ? la : rb, s1);
+            sts8<5>(z > 5 ? la : rb, s1 >> 8);
+            sts8<6>(z > 6 ? la : rb, s1 >> 16);
+            sts8<7>(z > 7 ? la : rb, s1 >> 24);
         } else {
+            if (st & 1u) sts8<0>(z > 0 ? la : rb, s0);
+            if (st & 2u) sts8<1>(z > 1 ? la : rb, s0 >> 8);
+            if (st & 4u) sts8<2>(z > 2 ? la : rb, s0 >> 16);
+            if (st & 8u) sts8<3>(z > 3 ? la : rb, s0 >> 24);
+            if (st & 16u) sts8<4>(z > 4 ? la : rb, s1);
+            if (st & 32u) sts8<5>(z > 5 ? la : rb, s1 >> 8);
+            if (st & 64u) sts8<6>(z > 6 ? la : rb, s1 >> 16);
+            if (st & 128u) sts8<7>(z > 7 ? la : rb, s1 >> 24);
+        }
+    }
+}
+
+// One side of a root window (its other child is a leaf): keep: the symbols
+// kept, one bit each; at: the place of the group's first kept symbol.
+__device__ inline void enc_keep(const EncSmem &S, uint32_t base, uint32_t keep, uint32_t at, const uint32_t (&y)[8]) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t sub = lane & 3, below = (1u << (8 * sub)) - 1u;
 #pragma unroll
-            for (int j = 0; j < 32; j++) {
-                const uint32_t bit = (bw >> j) & 1u;
-                const uint32_t val = (y[j >> 1] >> (16 * (j & 1))) << 1;
-                if ((uint32_t)j < vl) sts16(bit ? ra + ob : la + (2u * j - ob), val);
-                ob += 2u * bit;
+    for (int s = 0; s < 4; s++) {
+        const int own = 8 * s + (lane >> 2);
+        const uint32_t ws = __shfl_sync(0xffffffffu, keep, own), as = __shfl_sync(0xffffffffu, at, own);
+        const uint32_t p = base + as + __popc(ws & below), b8 = (ws >> (8 * sub)) & 0xFFu, c = __popc(b8);
+        const uint32_t e = S.lut[b8 ^ 0xFFu];
+        const uint32_t s0 = __byte_perm(y[2 * s], y[2 * s + 1], e);
+        if (c > 0) sts8<0>(p, s0);
+        if (c > 1) sts8<1>(p, s0 >> 8);
+        if (c > 2) sts8<2>(p, s0 >> 16);
+        if (c > 3) sts8<3>(p, s0 >> 24);
+        if (__any_sync(0xffffffffu, c > 4)) {   // (rare on the skewed roots that keep one side)
+            const uint32_t s1 = __byte_perm(y[2 * s], y[2 * s + 1], e >> 16);
+            if (c > 4) sts8<4>(p, s1);
+            if (c > 5) sts8<5>(p, s1 >> 8);
+            if (c > 6) sts8<6>(p, s1 >> 16);
+            if (c > 7) sts8<7>(p, s1 >> 24);
+        }
+    }
+}
+
+// code indices of four symbols; none: a byte of 255 among them
+__device__ inline uint32_t enc_codes4(const EncSmem &S, uint32_t x) {
+    return (uint32_t)S.ci[x & 0xFFu] | ((uint32_t)S.ci[(x >> 8) & 0xFFu] << 8) | ((uint32_t)S.ci[(x >> 16) & 0xFFu] << 16) |
+           ((uint32_t)S.ci[x >> 24] << 24);
+}
+__device__ inline uint32_t any255(uint32_t c) { return (~c - 0x01010101u) & c & 0x80808080u; }
+// 255 is a symbol's index only when all 256 have codes
+__device__ inline bool enc_all_codes(const EncSmem &S) {
+    return (S.pmask[0] & S.pmask[1] & S.pmask[2] & S.pmask[3] & S.pmask[4] & S.pmask[5] & S.pmask[6] & S.pmask[7]) ==
+           0xFFFFFFFFu;
+}
+
+// A warp packs 256 symbols of a flat node D bits each (the lane's 8 code
+// indices y0, y1, their first nv valid; lo4: the node's first code index in
+// all bytes) and writes the nbits packed bits at bit address a of the record:
+// words inside the run are stored, the two it shares with its neighbours are
+// ORed into the zeroed body.
+__device__ inline void enc_flat_step(uint32_t *strip, uint32_t *rec32, uint32_t D, uint32_t lo4, uint32_t y0, uint32_t y1,
+                                     int nv, uint32_t a, uint32_t nbits) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t m = (1u << D) - 1u;
+    auto pack = [&](uint32_t y, int n) {
+        const uint32_t x = (y - lo4) & mask4(n);   // (every valid byte is at least lo4's)
+        return (x & m) | ((x >> (8 - D)) & (m << D)) | ((x >> (16 - 2 * D)) & (m << (2 * D))) |
+               (D == 8 ? x & 0xFF000000u : (x >> (24 - 3 * D)) & (m << (3 * D)));
+    };
+    const uint64_t bits = (uint64_t)pack(y0, nv) | ((uint64_t)pack(y1, nv - 4) << (4 * D));
+    uint8_t *sb = reinterpret_cast<uint8_t *>(strip) + D * lane;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 8; k++)
+        if ((uint32_t)k < D) sb[k] = (uint8_t)(bits >> (8 * k));
+    __syncwarp();
+    const uint32_t sh = a & 31u, wi = a >> 5, end = sh + nbits;   // bits sh .. end - 1 of the words from wi on
+    for (uint32_t i = lane; 32 * i < end; i += 32) {
+        const uint32_t cur = 32 * i < nbits ? strip[i] : 0u, prev = i ? strip[i - 1] : 0u;
+        uint32_t o = sh ? (cur << sh) | (prev >> (32 - sh)) : cur;
+        if (32 * i + 32 > end) o &= (1u << (end - 32 * i)) - 1u;
+        if (32 * i >= sh && 32 * i + 32 <= end) rec32[wi + i] = o;
+        else if (o) atomicOr(&rec32[wi + i], o);
+    }
+}
+
+// One part of a block whose demands and cursors are in S: symbols [src, src +
+// C), every level; the whole CTA.  Ends with a barrier.
+__device__ inline void enc_part(EncSmem &S, const uint8_t *src, uint32_t C, const uint8_t *src_end, uint32_t *rec32) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint32_t sub = lane & 3;
+    uint32_t *strip = S.strip[warp];
+    uint8_t *stripb = reinterpret_cast<uint8_t *>(strip);
+    uint32_t par = 0;
+    // ---- the root: input bytes -> bits, code indices; children ----
+    {
+        const uint32_t chv = S.ch[0], rD = ch_flat_d(chv);
+        const uint32_t c0 = chv & 0xFFFFu, c1 = chv >> 16;
+        const bool i0 = !rD && !(c0 & 0x8000u), i1 = !rD && !(c1 & 0x8000u);
+        const uint32_t nwin = (C + kWin - 1) / kWin, mis = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 3);
+        // a leaf child decides the bit by its symbol alone; two internal ones (or a flat root) by the code index
+        const bool code = !rD && !(i0 && i1);
+        const uint32_t leaf4 = (i0 ? c1 & 0xFFu : c0 & 0xFFu) * 0x01010101u, flip = i0 ? 0u : 0xFFFFFFFFu;
+        const uint32_t split4v = S.split[0] * 0x01010101u;
+        const uint32_t base = smem_addr(S.buf[1]);
+        const uint32_t sp0 = i0 ? S.sp[c0 & 0xFFu] : 0u, sp1 = i1 ? S.sp[c1 & 0xFFu] : 0u;
+        const uint32_t dem0 = i0 ? S.dem[c0 & 0xFFu] : 0xFFFFFFFFu, dem1 = i1 ? S.dem[c1 & 0xFFu] : 0xFFFFFFFFu, pos0 = S.pos[0];
+        const bool al8 = !(reinterpret_cast<uintptr_t>(src) & 7);
+        uint32_t carry = 0;
+        bool bad = false;
+        for (uint32_t b0 = 0; b0 < nwin; b0 += kEncWarps) {
+            const uint32_t i = b0 + warp, k0 = kWin * i;
+            const bool full = k0 + kWin <= C;
+            uint32_t y[8], w = 0, inc = 0, pc = 0;
+            if (i < nwin) {
+                if (full && al8) {
+                    const uint2 *p = reinterpret_cast<const uint2 *>(src + k0) + lane;
+#pragma unroll
+                    for (int s = 0; s < 4; s++) {
+                        const uint2 x = __ldg(p + 32 * s);
+                        y[2 * s] = x.x;
+                        y[2 * s + 1] = x.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int s = 0; s < 4; s++) {
+                        const uint32_t k = k0 + 256 * s + 8 * lane;
+                        uint2 x = make_uint2(0u, 0u);
+                        if (k < C) x = ldg8(src + k, mis, src_end);
+                        y[2 * s] = x.x;
+                        y[2 * s + 1] = x.y;
+                    }
+                }
+                if (!code) {
+                    uint32_t none = 0;
+#pragma unroll
+                    for (int j = 0; j < 8; j++) {
+                        uint32_t c = enc_codes4(S, y[j]);
+                        if (!full) c &= mask4((int)C - (int)(k0 + 256 * (j >> 1) + 8 * lane + 4 * (j & 1)));
+                        none |= any255(c);
+                        y[j] = c;
+                    }
+                    if (none && !enc_all_codes(S)) bad = true;
+                } else if (!i0 && !i1) {   // two symbols in all: nothing else may occur
+#pragma unroll
+                    for (int j = 0; j < 8; j++) {
+                        const uint32_t ok = eq4(y[j] ^ leaf4) | eq4(y[j] ^ ((c1 & 0xFFu) * 0x01010101u));
+                        if (~ok & 0x80808080u & mask4((int)C - (int)(k0 + 256 * (j >> 1) + 8 * lane + 4 * (j & 1)))) bad = true;
+                    }
+                }
+                if (rD) {
+                    const uint32_t lo4 = split4v;
+#pragma unroll
+                    for (int s = 0; s < 4; s++) {
+                        const uint32_t k = k0 + 256 * s;
+                        if (k < C)
+                            enc_flat_step(strip, rec32, rD, lo4, y[2 * s], y[2 * s + 1],
+                                          max(0, min(8, (int)C - (int)(k + 8 * lane))), pos0 + k * rD, min(256u, C - k) * rD);
+                    }
+                } else {
+                    __syncwarp();
+#pragma unroll
+                    for (int s = 0; s < 4; s++) {
+                        uint32_t m0, m1;
+                        if (code) { m0 = eq4(y[2 * s] ^ leaf4) ^ flip; m1 = eq4(y[2 * s + 1] ^ leaf4) ^ flip; }
+                        else { m0 = ge4(y[2 * s], split4v); m1 = ge4(y[2 * s + 1], split4v); }
+                        stripb[32 * s + lane] = (uint8_t)gather8(m0, m1);
+                    }
+                    __syncwarp();
+                    const uint32_t kk = k0 + kGrp * lane, vl = full ? 32u : (kk < C ? min(32u, C - kk) : 0u);
+                    w = strip[lane];
+                    if (vl < 32) w &= (1u << vl) - 1u;
+                    pc = __popc(w);
+                    inc = warp_inclusive(pc);
+                    if (lane == 31) S.wtot[par][warp] = inc;
+                    inc -= pc;
+                    enc_put_bits(rec32, vl != 0, 0u, pos0 + kk, w, vl);
+                }
+            }
+            __syncthreads();
+            if (!rD) {
+                // ones before each window of the round (lane: window)
+                const uint32_t x = lane < kEncWarps && b0 + lane < nwin ? S.wtot[par][lane] : 0u;
+                uint32_t in = x;
+#pragma unroll
+                for (int o = 1; o < kEncWarps; o <<= 1) {
+                    const uint32_t z = __shfl_up_sync(0xffffffffu, in, o);
+                    if (lane >= o) in += z;
+                }
+                const uint32_t r1 = carry + __shfl_sync(0xffffffffu, in - x, warp) + inc;
+                carry += __shfl_sync(0xffffffffu, in, kEncWarps - 1);
+                if (i < nwin) {
+                    const uint32_t kk = k0 + kGrp * lane, vl = full ? 32u : (kk < C ? min(32u, C - kk) : 0u);
+                    // a part whose symbols do not match its counts must not write past the spans
+                    const bool over = vl && (r1 + pc > dem1 || kk + vl - r1 - pc > dem0);
+                    if (over) bad = true;
+                    if (code) {
+                        const uint32_t vm = vl >= 32 ? 0xFFFFFFFFu : (1u << vl) - 1u;
+                        if (i0 || i1) enc_keep(S, base, over ? 0u : (i0 ? ~w : w) & vm, i0 ? sp0 + kk - r1 : sp1 + r1, y);
+                    } else {
+                        EncGrp G;
+                        G.w = w;
+                        G.a = over ? 0u : (sp0 + kk - r1) | ((sp1 + r1) << 16);
+                        G.b = (over ? 0u : vl) | 0xC0u;
+                        enc_partition(S, base, G, y);
+                    }
+                }
+            }
+            par ^= 1u;
+        }
+        if (code && (i0 || i1)) {
+            // the kept symbols are input bytes still: their code indices
+            __syncthreads();
+            const uint32_t n1 = S.dem[i0 ? c0 & 0xFFu : c1 & 0xFFu];
+            uint2 *p = reinterpret_cast<uint2 *>(S.buf[1] + (i0 ? sp0 : sp1));
+            uint32_t none = 0;
+            for (uint32_t k = 8 * t; k < n1; k += 8 * kEncThreads) {
+                uint2 x = p[k >> 3];
+                x.x = enc_codes4(S, x.x);
+                x.y = enc_codes4(S, x.y);
+                p[k >> 3] = x;
+                none |= any255(x.x & mask4((int)(n1 - k))) | any255(x.y & mask4((int)(n1 - k) - 4));
+            }
+            if (none && !enc_all_codes(S)) bad = true;
+        }
+        if (bad) S.bad = 1;
+    }
+    __syncthreads();
+    // ---- depths 1.. : node spans of buf[d & 1] into the children's spans ----
+    for (int d = 1; d < (int)S.maxd; d++) {
+        const uint8_t *bin = S.buf[d & 1];
+        const uint32_t base = smem_addr(S.buf[(d + 1) & 1]);
+        const uint32_t nw = S.nw[d], nwo = S.nwo[d], wn = S.wn_off[d], f0 = S.first[d];
+        uint32_t carry = 0;
+        bool bad = false;
+        for (uint32_t b0 = 0; b0 < nw; b0 += kEncWarps) {
+            const uint32_t i = b0 + warp;
+            uint32_t v = 0, q = 0, left = 0, y[8], w = 0, inc = 0, pc = 0;
+            if (i < nwo) {
+                left = lvl_locate(S, d, wn, f0, i, v, q);
+                // bits 0..15: the group's place in the level buffer, 16..23: the node's split
+                const uint32_t pk = (left ? (uint32_t)S.sp[v] + kGrp * q : 0u) | ((uint32_t)S.split[v] << 16);
+                __syncwarp();
+#pragma unroll
+                for (int s = 0; s < 4; s++) {
+                    const uint32_t ps = __shfl_sync(0xffffffffu, pk, 8 * s + (lane >> 2));
+                    const uint2 x = *reinterpret_cast<const uint2 *>(bin + (ps & 0xFFFFu) + 8 * sub);
+                    const uint32_t sv = (ps >> 16) * 0x01010101u;
+                    y[2 * s] = x.x;
+                    y[2 * s + 1] = x.y;
+                    stripb[32 * s + lane] = (uint8_t)gather8(ge4(x.x, sv), ge4(x.y, sv));
+                }
+                __syncwarp();
+                w = left ? strip[lane] : 0u;
+                if (left < 32) w &= (1u << left) - 1u;
+                pc = __popc(w);
+                inc = warp_inclusive(pc);
+                if (lane == 31) S.wtot[par][warp] = inc;
+                inc -= pc;
+                // a node's first group: the ones of the window before it
+                if (q == 0) S.fw[v] = (uint16_t)inc;
+                enc_put_bits(rec32, left != 0, v, S.pos[v] + kGrp * q, w, min(32u, left));
+            }
+            __syncthreads();
+            par ^= 1u;
+            if (i < nwo) {
+                uint32_t ex = 0, ps = 0;
+                if (nwo > 1) {
+                    // ones of the level before each window of the round (lane: window)
+                    const uint32_t x = lane < kEncWarps && b0 + lane < nwo ? S.wtot[par ^ 1u][lane] : 0u;
+                    uint32_t in = x;
+#pragma unroll
+                    for (int o = 1; o < kEncWarps; o <<= 1) {
+                        const uint32_t z = __shfl_up_sync(0xffffffffu, in, o);
+                        if (lane >= o) in += z;
+                    }
+                    ex = carry + in - x;
+                    if (nwo > kEncWarps) {
+                        carry += __shfl_sync(0xffffffffu, in, kEncWarps - 1);
+                        if (warp == 0 && lane < kEncWarps && b0 + lane < nwo) S.wpre[wn + b0 + lane] = (uint16_t)ex;
+                    }
+                    // at the node's first group
+                    const uint32_t gw = (32u * i + lane - q) >> 5;   // its window
+                    ps = __shfl_sync(0xffffffffu, ex, gw - b0);
+                    if (gw < b0) ps = S.wpre[wn + gw];
+                    ex = __shfl_sync(0xffffffffu, ex, warp);
+                }
+                const uint32_t r1 = (ex + inc - ps - S.fw[v]) & 0xFFFFu, kk = kGrp * q, vl = min(32u, left);
+                const uint32_t chv = S.ch[v], c0 = chv & 0xFFFFu, c1 = chv >> 16;
+                const bool i0 = left && !(c0 & 0x8000u), i1 = left && !(c1 & 0x8000u);
+                const bool over = (i1 && r1 + pc > S.dem[c1 & 0xFFu]) || (i0 && kk + vl - r1 - pc > S.dem[c0 & 0xFFu]);
+                if (over) bad = true;
+                EncGrp G;
+                G.w = w;
+                G.a = over ? 0u : (((i0 ? (uint32_t)S.sp[c0 & 0xFFu] : 0u) + kk - r1) & 0xFFFFu) |
+                                      (((i1 ? (uint32_t)S.sp[c1 & 0xFFu] : 0u) + r1) << 16);
+                G.b = (over ? 0u : vl) | (i0 ? 0x40u : 0u) | (i1 ? 0x80u : 0u);
+                enc_partition(S, base, G, y);
+            } else if (i < nw) {
+                // a flat node's window: its packed indices
+                const uint32_t v2 = S.wnode[wn + i], fD = ch_flat_d(S.ch[v2]), dv = S.dem[v2], lo4 = S.split[v2] * 0x01010101u;
+                const uint32_t k0 = (i - nwo - S.fw[v2]) * kWin, k1 = min(dv, k0 + kWin);
+#pragma unroll 1
+                for (uint32_t k = k0; k < k1; k += 256) {
+                    const uint32_t kl = k + 8 * lane;
+                    uint2 x = make_uint2(0u, 0u);
+                    if (kl < dv) x = *reinterpret_cast<const uint2 *>(bin + S.sp[v2] + kl);
+                    enc_flat_step(strip, rec32, fD, lo4, x.x, x.y, max(0, min(8, (int)dv - (int)kl)), S.pos[v2] + k * fD,
+                                  min(256u, dv - k) * fD);
+                }
             }
         }
-    } else if (i0 || i1) {
-        // one side: its symbols are the set bits of m, stored in order
-        const uint32_t m = (i1 ? bw : ~bw) & vm;
-        uint32_t a = i1 ? ra : la;
-#pragma unroll
-        for (int j = 0; j < 32; j++) {
-            const uint32_t val = (y[j >> 1] >> (16 * (j & 1))) << 1;
-            if ((m >> j) & 1u) sts16(a, val);
-            a += 2u * ((m >> j) & 1u);
-        }
+        if (bad) S.bad = 1;
+        __syncthreads();
     }
 }
 
-// Packs the top D bits of the 16-bit values y (value j in half j & 1 of
-// y[j >> 1]; the first vl valid) D bits per value, value j at bits [jD,
-// jD + D) (Sec. 2.2.3 packed indices, App. D), and writes the vl D bits at
-// bit address a of the record: words inside the run are stored, the two it
-// shares with its neighbours are ORed into the zeroed body.
-template <int D>
-__device__ inline void flat_emit(uint32_t *rec32, uint32_t a, const uint32_t (&y)[16], uint32_t vl) {
-    uint32_t w[D];
-#pragma unroll
-    for (int k = 0; k < D; k++) w[k] = 0;
-#pragma unroll
-    for (int j = 0; j < 32; j++) {
-        const uint32_t x = (uint32_t)j < vl ? ((y[j >> 1] >> (16 * (j & 1))) & 0xFFFFu) >> (16 - D) : 0u;
-        const int b = j * D, wi = b >> 5, sh = b & 31;
-        w[wi] |= x << sh;
-        if (sh + D > 32) w[wi + 1] |= x >> (32 - sh);
-    }
-    const uint32_t sh = a & 31u, wi = a >> 5, end = sh + vl * (uint32_t)D;
-    uint32_t prev = 0;
-#pragma unroll
-    for (int k = 0; k <= D; k++) {
-        const uint32_t cur = k < D ? w[k] : 0u;
-        const uint32_t o = sh ? (cur << sh) | (prev >> (32 - sh)) : cur;
-        prev = cur;
-        const uint32_t lo = 32u * (uint32_t)k;
-        if (lo < end) {
-            if (lo >= sh && lo + 32u <= end) rec32[wi + k] = o;
-            else if (o) atomicOr(&rec32[wi + k], o);
-        }
+// Counts input bytes [lo, hi) of the block at src into hist (288 zeroed bins;
+// the whole CTA, no barrier).
+__device__ inline void enc_count(const uint8_t *src, uint32_t lo, uint32_t hi, const uint8_t *src_end, uint32_t *hist,
+                                 uint32_t hot) {
+    for (uint32_t kb = lo + 32u * threadIdx.x; kb < hi; kb += 32u * kEncThreads) {
+        uint32_t x[8];
+        ldg32(src + kb, src_end, x);
+        hist_add32(hist, x, min(32u, hi - kb), hot);
     }
 }
 
-__device__ inline void flat_emit_d(uint32_t D, uint32_t *rec32, uint32_t a, const uint32_t (&y)[16], uint32_t vl) {
-    switch (D) {
-        case 2: flat_emit<2>(rec32, a, y, vl); break;
-        case 3: flat_emit<3>(rec32, a, y, vl); break;
-        case 4: flat_emit<4>(rec32, a, y, vl); break;
-        case 5: flat_emit<5>(rec32, a, y, vl); break;
-        case 6: flat_emit<6>(rec32, a, y, vl); break;
-        case 7: flat_emit<7>(rec32, a, y, vl); break;
-        default: flat_emit<8>(rec32, a, y, vl); break;
-    }
-}
-
-// Codes plan chunks cA .. cB - 1 of block b with the whole CTA (every
-// thread calls it with the same arguments).  whole: the block entire, its
-// header written, its body zeroed here and its status written; else one
-// chunk of a big block: the reset pass has checked the block, zeroed its
-// body and set its status, the chunk starts at the node cursors the counts
-// of the chunks before it give, chunk 0 writes the header and tables, and
-// the status only ever turns to an error.
-template <bool whole, typename SM>
-__device__ inline void encode_item(int b, uint32_t cA, uint32_t cB, const uint8_t *__restrict__ in,
+// Codes block b with the whole CTA (every thread calls it with the same
+// arguments).  whole: the block entire, its header written, its body zeroed
+// here and its status written; else share `share` of `shares` of plan chunk
+// cA of a big block: the reset pass has checked the block, zeroed its body
+// and set its status, the share starts at the node cursors the counts of the
+// chunks before it (and of the chunk's symbols before the share, counted
+// here) give, the first item writes the header and tables, and the status
+// only ever turns to an error.
+template <bool whole>
+__device__ inline void encode_item(int b, uint32_t cA, uint32_t share, uint32_t shares, const uint8_t *__restrict__ in,
                                    const uint64_t *__restrict__ blk_off, const BlockLayout *__restrict__ layout,
                                    const uint32_t *__restrict__ chunk_hist, uint8_t *__restrict__ out,
                                    const uint64_t *__restrict__ out_off, uint64_t *__restrict__ rec_bytes,
-                                   int32_t *__restrict__ status, SM &S) {
+                                   int32_t *__restrict__ status, EncSmem &S) {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const uint64_t i0 = blk_off[b], i1 = blk_off[b + 1], o0 = out_off[b], o1 = out_off[b + 1];
-    const uint32_t nw = enc_nchunks(i1 - i0), cEnd = cB < nw ? cB : nw;
+    const uint64_t n = i1 - i0;
+    const uint32_t nw = enc_nchunks(n);
+    // the item's symbols: whole multiples of 32 but for the block's end
+    const uint32_t ch0 = whole ? 0u : enc_chunk_start(n, cA, nw), ch1 = whole ? (uint32_t)n : enc_chunk_start(n, cA + 1, nw);
+    const uint32_t P0 = ch0 + (uint32_t)((uint64_t)(ch1 - ch0) * share / shares & ~31ull);
+    const uint32_t P1 = share + 1 == shares ? ch1 : ch0 + (uint32_t)((uint64_t)(ch1 - ch0) * (share + 1) / shares & ~31ull);
     // the item's input is read by the root pass: ask L2 for it now, so
     // those reads find it there
     {
-        const uint64_t lo = enc_chunk_start(i1 - i0, cA, nw), hi = enc_chunk_start(i1 - i0, cEnd, nw);
-        const uint8_t *p0 = in + i0 + lo;
-        for (uint64_t i = 128ull * t; i < hi - lo; i += 128ull * kEncThreads)
+        const uint8_t *p0 = in + i0 + P0;
+        for (uint64_t i = 128ull * t; i < P1 - P0; i += 128ull * kEncThreads)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(p0 + i));
     }
     // the block's layout, staged into shared memory once (coalesced); it
@@ -417,7 +638,6 @@ __device__ inline void encode_item(int b, uint32_t cA, uint32_t cB, const uint8_
     }
     __syncthreads();
     const BlockLayout &L = *reinterpret_cast<const BlockLayout *>(S.buf[1]);
-    const uint64_t n = i1 - i0;
     uint8_t *rec = out + o0;
     const uint64_t cap = o1 - o0;
     const uint32_t kind = L.kind;
@@ -431,7 +651,7 @@ __device__ inline void encode_item(int b, uint32_t cA, uint32_t cB, const uint8_
     }
     const int V = L.n_int;
     const uint32_t rec_bound = L.rec_bound;   // the staged layout is overwritten once the levels start
-    const bool head = whole || cA == 0;   // this item writes the header and tables
+    const bool head = whole || (cA == 0 && share == 0);   // this item writes the header and tables
     // ---- record header (App. D, adapted) ----
     if (t < 16 && head) {
         uint8_t v = 0;
@@ -485,42 +705,65 @@ __device__ inline void encode_item(int b, uint32_t cA, uint32_t cB, const uint8_
     // ---- per-block tables ----
     {
         const uint32_t l = L.len[t];
-        S.code16[t] = l ? (uint16_t)((uint32_t)L.code[t] << (16 - l)) : 0;
+        if (!l) S.ci[t] = 255;
         if (t < V) {
             uint32_t code2 = 0;
             for (int c = 0; c < 2; c++) {
                 const int ch = L.child[t][c];
                 code2 |= (ch >= 0 ? (uint32_t)ch : (0x8000u | (uint32_t)(-ch - 1))) << (16 * c);
             }
-            S.ch[t] = L.fd[t] ? ch_flat(L.fd[t], L.fbase[t]) : code2;
-            S.bitsrc[t] = 8u * L.body_off[t];
+            const uint32_t fd = L.fd[t];
+            S.ch[t] = fd ? ch_flat(fd, L.fbase[t]) : code2;
             S.pos[t] = 8u * L.body_off[t];
-            S.nv[t] = L.nv[t] * max(1u, (uint32_t)L.fd[t]);
+            S.end[t] = 8u * L.body_off[t] + L.nv[t] * max(1u, fd);
         }
         if (t < 17) S.first[t] = L.depth_first[t];
         if (t == 0) { S.maxd = L.max_depth; S.hot = 0xFFFFu; S.bad = 0; }
+        {   // byte t: zeros to the front, both sides in order
+            uint32_t e = 0, z = 0, o = 8u - __popc((uint32_t)t);
+            for (uint32_t j = 0; j < 8; j++) {
+                const uint32_t k = ((uint32_t)t >> j) & 1u ? o++ : z++;
+                e |= j << (4 * k);
+            }
+            S.lut[t] = e;
+        }
     }
     __syncthreads();
+    const uint32_t part = max(1024u, L.part);
+    const bool big = L.big != 0;
     {
         const uint32_t l = L.len[t];
         const uint32_t key = __reduce_min_sync(0xffffffffu, l ? (l << 8) | (uint32_t)t : 0xFFFFu);
         if (lane == 0) atomicMin(&S.hot, key);
         const uint32_t pm = __ballot_sync(0xffffffffu, l != 0);
         if (lane == 0) S.pmask[warp] = pm;
+        // a node's bit is one from its right child's first code index on
+        if (t < V) {
+            const uint32_t chv = S.ch[t], c1 = chv >> 16;
+            S.split[t] = ch_flat_d(chv) ? S.nlo[t] : (c1 & 0x8000u ? S.ci[c1 & 0xFFu] : S.nlo[c1 & 0xFFu]);
+        }
     }
     __syncthreads();   // (the staged layout is dead from here on)
     const uint32_t hot = S.hot & 0xFFu;
     const uint8_t *src = in + i0;
     const uint8_t *src_end = in + i1;
     uint32_t *rec32 = reinterpret_cast<uint32_t *>(rec);
-    // counting scratch in the second level buffer (free between chunks)
+    // counting scratch in the second level buffer (free between parts)
     uint32_t *hist = reinterpret_cast<uint32_t *>(S.buf[1]);
     uint32_t *hc = hist + 288, *ps = hist + 544;   // (after the 32 lane bins of the counting)
-    // a chunk of a big block starts every node's cursor after the symbols
-    // the chunks before it put there
-    if (cA > 0) {
-        uint32_t h = 0;
+    uint32_t acc = 0;              // count of symbol t in the plan chunk's symbols counted so far
+    // an item inside a block starts every node's cursor after the symbols before it
+    if (!whole && (cA > 0 || share > 0)) {
+        for (int s = t; s < 288; s += kEncThreads) hist[s] = 0;
+        __syncthreads();
+        enc_count(src, ch0, P0, src_end, hist, hot);
+        __syncthreads();
+        if (warp == 0) hist_fold_hot(hist, hot);
+        __syncthreads();
+        uint32_t h = hist[t];
+        acc = h;
         for (uint32_t c = 0; c < cA; c++) h += __ldg(chunk_hist + ((size_t)b * kEncChunks + c) * 256 + t);
+        __syncthreads();
         hist[t] = h;
         __syncthreads();
         if (warp == 0) enc_counts(S, hist, S.dem, hc, ps);
@@ -528,284 +771,77 @@ __device__ inline void encode_item(int b, uint32_t cA, uint32_t cB, const uint8_
         if (t < V) S.pos[t] += S.dem[t] * max(1u, ch_flat_d(S.ch[t]));
         __syncthreads();
     }
-    // ---- chunks: runs of the planning pass's chunks, or parts of one ----
-    uint32_t c0 = cA, k = cEnd - cA;    // the run of plan chunks tried: c0 .. c0 + k - 1
-    uint32_t P = enc_chunk_start(n, cA, nw), sub = 0;   // sub > 0: cutting plan chunk c0 into parts of `sub` symbols
-    const uint32_t Pend = enc_chunk_start(n, cEnd, nw);
-    uint32_t acc = 0;              // count of symbol t in the coded parts of plan chunk c0
-    while (P < Pend) {
-        const uint32_t Q1 = enc_chunk_start(n, c0 + (sub ? 1u : k), nw);   // end of the run / plan chunk
-        const uint32_t C = sub ? min(sub, Q1 - P) : Q1 - P;
-        // the chunk's histogram: the planning pass's chunk counts, or counted here
-        for (int s2 = t; s2 < 256 + 32; s2 += kEncThreads) hist[s2] = 0;
+    // ---- parts ----
+    uint32_t P = P0, len = whole && !(big && !chunk_hist) ? P1 - P0 : part;
+    while (P < P1) {
+        const uint32_t C = min(len, P1 - P);
+        // the part's histogram: the planning pass's chunk counts, or counted here
+        for (int s = t; s < 288; s += kEncThreads) hist[s] = 0;
         __syncthreads();
-        if (chunk_hist && !sub) {
+        const bool given = whole && chunk_hist && C == P1 - P0;
+        if (given) {
             uint32_t h = 0;
-            for (uint32_t c = c0; c < c0 + k; c++) h += __ldg(chunk_hist + ((size_t)b * kEncChunks + c) * 256 + t);
+            for (uint32_t c = 0; c < nw; c++) h += __ldg(chunk_hist + ((size_t)b * kEncChunks + c) * 256 + t);
             hist[t] = h;
         } else {
-            for (uint32_t kb = P + 32u * t; kb < P + C; kb += 32u * kEncThreads) {
-                uint32_t x[8];
-                ldg32(src + kb, src_end, x);
-                hist_add32(hist, x, min(32u, P + C - kb), hot);
-            }
+            enc_count(src, P, P + C, src_end, hist, hot);
             __syncthreads();
             if (warp == 0) hist_fold_hot(hist, hot);
         }
         __syncthreads();
         const uint32_t hcount = hist[t];
         if (warp == 0) {
-            // the counts must total the chunk, with no symbol the code lacks
+            // the counts must total the part, with no symbol the code lacks
             uint32_t tot = 0, nocode = 0;
-            for (int s2 = lane; s2 < 256; s2 += 32) {
-                tot += hist[s2];
-                if (hist[s2] && !((S.pmask[s2 >> 5] >> (s2 & 31)) & 1u)) nocode = 1;
+            for (int s = lane; s < 256; s += 32) {
+                tot += hist[s];
+                if (hist[s] && !((S.pmask[s >> 5] >> (s & 31)) & 1u)) nocode = 1;
             }
             tot = __reduce_add_sync(0xffffffffu, tot);
             if (__any_sync(0xffffffffu, nocode) || tot != C) { if (lane == 0) S.bad = 1; }
             else enc_counts(S, hist, S.dem, hc, ps);
-            if (lane == 0) { S.fits = 1; S.lvl_max = 0; }
         }
         __syncthreads();
         if (S.bad) break;
-        // no node's bits of this chunk may run past its body (counts that do
+        // no node's bits of this part may run past its body (counts that do
         // not describe the input could otherwise carry a cursor beyond it)
-        if (t < V && (uint64_t)S.pos[t] + (uint64_t)S.dem[t] * max(1u, ch_flat_d(S.ch[t])) >
-                         (uint64_t)S.bitsrc[t] + S.nv[t])
-            S.bad = 1;
-        __syncthreads();
-        if (S.bad) break;
-        for (int d = warp; d < (int)S.maxd; d += kEncWarps)
-            if (!enc_layout_level(S, d) && lane == 0) S.fits = 0;
-        __syncthreads();
-        const bool fits = S.fits != 0;
-        __syncthreads();
-        if (!fits) {
-            // a shorter run of plan chunks, or parts of one chunk (32 symbols
-            // always fit: a level then holds at most 32 symbols in 160 groups)
-            if (sub == 32u) {
+        if (__syncthreads_or(t < V && (uint64_t)S.pos[t] + (uint64_t)S.dem[t] * max(1u, ch_flat_d(S.ch[t])) > S.end[t])) {
+            if (t == 0) S.bad = 1;
+            break;
+        }
+        if (!lvl_layout(S)) {
+            // a shorter part (32 symbols always fit: a level then holds at
+            // most 32 symbols in 160 groups)
+            if (C <= 32u) {
                 if (t == 0) S.bad = 1;
                 break;
             }
-            if (!sub && k > 1) {
-                k = (k + 1) / 2;
-            } else {
-                // parts whose largest level fills at most 7/8 of a buffer,
-                // scaled from this try's largest level, and at least halved
-                const uint32_t cur = sub ? sub : C, lm = S.lvl_max;
-                const uint32_t est = lm ? (uint32_t)((uint64_t)cur * (SM::kBuf - SM::kBuf / 8) / lm) : cur / 2;
-                sub = max(32u, min(cur / 2, est) & ~31u);
-            }
+            len = max(32u, (len > part ? part : len / 2) & ~31u);
             continue;
         }
-        // ---- the root: input bytes -> codes; bits; children ----
-        uint32_t par = 0;
-        if (const uint32_t rD = ch_flat_d(S.ch[0])) {
-            // a flat root (the whole alphabet one group): the packed indices
-            for (uint32_t kk = 32u * t; kk < C; kk += 32u * kEncThreads) {
-                uint32_t x[8];
-                ldg32(src + P + kk, src_end, x);
-                uint32_t y[16];
-#pragma unroll
-                for (int j = 0; j < 16; j++) {
-                    const uint32_t s0 = (x[j >> 1] >> (16 * (j & 1))) & 0xFFu, s1 = (x[j >> 1] >> (16 * (j & 1) + 8)) & 0xFFu;
-                    y[j] = (uint32_t)S.code16[s0] | ((uint32_t)S.code16[s1] << 16);
-                }
-                flat_emit_d(rD, rec32, S.pos[0] + kk * rD, y, min(32u, C - kk));
-            }
-        } else {
-            const uint32_t chv = S.ch[0], c0n = chv & 0xFFFFu, c1n = chv >> 16;
-            const bool i0c = !(c0n & 0x8000u), i1c = !(c1n & 0x8000u);
-            const uint32_t nb = smem_addr(S.buf[1]);
-            const uint32_t lp0 = nb + 2u * (i0c ? S.sp[c0n & 0xFFu] : 0u), rp0 = nb + 2u * (i1c ? S.sp[c1n & 0xFFu] : 0u);
-            const uint32_t G = (C + 31) >> 5;
-            uint32_t rc = 0;
-            // the next round's 32 bytes of each lane are loaded while this one is coded
-            uint32_t xn[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            if (32u * (32u * warp + lane) < C) ldg32(src + P + 32u * (32u * warp + lane), src_end, xn);
-            for (uint32_t r0 = 0; r0 < G; r0 += 32 * kEncWarps) {
-                const uint32_t kk = 32u * (r0 + 32u * warp + lane);
-                const bool act = kk < C;
-                const uint32_t vl = act ? min(32u, C - kk) : 0u;
-                uint32_t x[8];
-#pragma unroll
-                for (int q = 0; q < 8; q++) { x[q] = xn[q]; xn[q] = 0u; }
-                if (kk + 32u * 32u * kEncWarps < C) ldg32(src + P + kk + 32u * 32u * kEncWarps, src_end, xn);
-                uint32_t y[16];
-#pragma unroll
-                for (int j = 0; j < 16; j++) {
-                    const uint32_t s0 = (x[j >> 1] >> (16 * (j & 1))) & 0xFFu, s1 = (x[j >> 1] >> (16 * (j & 1) + 8)) & 0xFFu;
-                    y[j] = (uint32_t)S.code16[s0] | ((uint32_t)S.code16[s1] << 16);
-                }
-                uint32_t bw = top_bits8(y[0], y[1], y[2], y[3]) | (top_bits8(y[4], y[5], y[6], y[7]) << 8) |
-                              (top_bits8(y[8], y[9], y[10], y[11]) << 16) |
-                              (top_bits8(y[12], y[13], y[14], y[15]) << 24);
-                if (vl < 32) bw &= (1u << vl) - 1u;
-                const uint32_t pc = __popc(bw);
-                uint32_t inc = pc;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t yy = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += yy;
-                }
-                if (lane == 31) S.win[par][warp] = EncWin{inc, 0u};
-                __syncthreads();
-                uint32_t cin;
-                {
-                    const uint32_t ws = lane < kEncWarps ? S.win[par][lane].sum : 0u;
-                    uint32_t wi = ws;
-#pragma unroll
-                    for (int o = 1; o < kEncWarps; o <<= 1) {
-                        const uint32_t yy = __shfl_up_sync(0xffffffffu, wi, o);
-                        if (lane >= o) wi += yy;
-                    }
-                    cin = rc + __shfl_sync(0xffffffffu, wi - ws, warp);
-                    rc += __shfl_sync(0xffffffffu, wi, kEncWarps - 1);
-                }
-                par ^= 1u;
-                const uint32_t r1 = cin + inc - pc;
-                enc_put_bits(rec32, act, 0u, S.pos[0] + kk, bw, vl);
-                // a chunk whose symbols do not match its counts must not write past the spans
-                if (act && ((i1c && r1 + pc > S.dem[c1n & 0xFFu]) || (i0c && kk + vl - r1 - pc > S.dem[c0n & 0xFFu])))
-                    S.bad = 1;
-                else if (act) enc_split(lp0 + 2u * (kk - r1), rp0 + 2u * r1, i0c, i1c, y, bw, vl);
-            }
-        }
-        __syncthreads();
-        // ---- depths 1.. : node spans of buf[d & 1] into the children's spans ----
-        for (int d = 1; d < (int)S.maxd; d++) {
-            const uint16_t *bin = S.buf[d & 1];
-            uint16_t *bout = S.buf[(d + 1) & 1];
-            const uint32_t f1 = S.first[d + 1], G = S.lg[d];
-            const uint32_t le = 0xFFFFFFFFu >> (31 - lane);
-            uint32_t rc_sum = 0;
-            for (uint32_t r0 = 0; r0 < G; r0 += 32 * kEncWarps) {
-                const uint32_t base = r0 + 32u * warp;
-                if (base >= G) {
-                    // past the level's end (its last round only): an empty
-                    // summary and nothing to code
-                    if (lane == 0) S.win[par][warp] = EncWin{0u, 0u};
-                    __syncthreads();
-                    par ^= 1u;
-                    continue;
-                }
-                // this warp's window: the node of each group
-                uint32_t v = 0, kk = 0, dv = 0, starts = 0;
-                bool act = false;
-                if (base < G) {
-                    const uint32_t u = S.wnode[d][base >> 5];
-                    const uint32_t vcur = (uint32_t)S.gs[u] == base ? u - 1 : u;
-                    const uint32_t cand = vcur + 1 + lane;
-                    uint32_t bit = 0;
-                    if (cand < f1) {
-                        const uint32_t sd = (uint32_t)S.gs[cand] - base;
-                        if (sd < 32) bit = 1u << sd;
-                    }
-                    starts = __reduce_or_sync(0xffffffffu, bit);
-                    v = vcur + __popc(starts & le);
-                    const uint32_t g = base + lane;
-                    kk = (g - S.gs[v]) * 32u;
-                    dv = S.dem[v];
-                    act = g < G && kk < dv;
-                }
-                const uint32_t vl = act ? min(32u, dv - kk) : 0u;
-                uint32_t y[16];
-                if (act) {
-                    // 16-byte loads: four per lane instead of sixteen, and four
-                    // times fewer shared-memory wavefronts for the same bytes
-                    const uint4 *p = reinterpret_cast<const uint4 *>(bin + S.sp[v] + kk);
-#pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        const uint4 u = p[q];
-                        y[4 * q] = u.x; y[4 * q + 1] = u.y; y[4 * q + 2] = u.z; y[4 * q + 3] = u.w;
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; j++) y[j] = 0;
-                }
-                const uint32_t fD = act ? ch_flat_d(S.ch[v]) : 0u;   // a flat node's lanes have no ranks
-                uint32_t bw = top_bits8(y[0], y[1], y[2], y[3]) | (top_bits8(y[4], y[5], y[6], y[7]) << 8) |
-                              (top_bits8(y[8], y[9], y[10], y[11]) << 16) |
-                              (top_bits8(y[12], y[13], y[14], y[15]) << 24);
-                if (vl < 32) bw &= (1u << vl) - 1u;
-                if (fD) bw = 0;
-                const uint32_t pc = __popc(bw);
-                uint32_t inc = pc;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t yy = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += yy;
-                }
-                const uint32_t sl = starts & le;
-                const int s0 = sl ? 31 - __clz(sl) : -1;
-                const uint32_t before = __shfl_sync(0xffffffffu, inc, s0 > 0 ? s0 - 1 : 0);
-                uint32_t r1 = inc - pc - (s0 > 0 ? before : 0u);
-                // a level of one window (warp 0's, in the first round) takes no carry
-                const bool one = G <= 32;
-                if (lane == 31 && !one)
-                    S.win[par][warp] = EncWin{r1 + pc, (starts & 1u) | (starts ? 2u : 0u) | (base < G ? 4u : 0u)};
-                __syncthreads();
-                const uint32_t cin = one ? 0u : enc_round_carry(S, par, rc_sum);
-                par ^= 1u;
-                if (s0 < 0) r1 += cin;   // groups of the node that runs in from the window before
-                enc_put_bits(rec32, act && !fD, v, S.pos[v] + kk, bw, vl);
-                if (act && fD) {
-                    flat_emit_d(fD, rec32, S.pos[v] + kk * fD, y, vl);
-                } else if (act) {
-                    const uint32_t chv = S.ch[v], c0n = chv & 0xFFFFu, c1n = chv >> 16;
-                    const bool i0c = !(c0n & 0x8000u), i1c = !(c1n & 0x8000u);
-                    const uint32_t ob = smem_addr(bout);
-                    const uint32_t lp = ob + 2u * ((i0c ? S.sp[c0n & 0xFFu] : 0u) + (kk - r1));
-                    const uint32_t rp = ob + 2u * ((i1c ? S.sp[c1n & 0xFFu] : 0u) + r1);
-                    if ((i1c && r1 + pc > S.dem[c1n & 0xFFu]) || (i0c && kk + vl - r1 - pc > S.dem[c0n & 0xFFu]))
-                        S.bad = 1;
-                    else
-                        enc_split(lp, rp, i0c, i1c, y, bw, vl);
-                }
-            }
-            __syncthreads();
-        }
+        enc_part(S, src + P, C, src_end, rec32);
         if (t < V) S.pos[t] += S.dem[t] * max(1u, ch_flat_d(S.ch[t]));
         __syncthreads();
         if (S.bad) break;
         P += C;
-        if (sub) {
-            acc += hcount;
-            if (P >= Q1) {
-                // plan chunk done in parts: its given counts must be the ones just counted
-                if (__syncthreads_or(chunk_hist && acc != __ldg(chunk_hist + ((size_t)b * kEncChunks + c0) * 256 + t))) {
-                    if (t == 0) S.bad = 1;
-                    break;
-                }
-                acc = 0;
-                sub = 0;   // whole runs again
-                c0 += 1;
-                k = cEnd - c0;
-            }
-        } else {
-            c0 += k;
-            k = cEnd - c0;
-        }
+        acc += hcount;
+        if (len < part) len = min(part, 2 * len);
     }
     __syncthreads();
-    // a chunk of a big block ends where the next one starts: the cursors
-    // after the symbols of chunks 0 .. cEnd - 1
-    if (cEnd < nw && !S.bad) {
-        uint32_t h = 0;
-        for (uint32_t c = 0; c < cEnd; c++) h += __ldg(chunk_hist + ((size_t)b * kEncChunks + c) * 256 + t);
-        hist[t] = h;
-        __syncthreads();
-        if (warp == 0) enc_counts(S, hist, S.dem, hc, ps);
-        __syncthreads();
-        if (t < V) S.nv[t] = S.pos[t] == S.bitsrc[t] + S.dem[t] * max(1u, ch_flat_d(S.ch[t])) ? S.pos[t] - S.bitsrc[t]
-                                                                                             : 0xFFFFFFFFu;
+    if (!whole && !S.bad) {
+        // the chunk's given counts must be the ones counted; an item inside
+        // the block ends where the next one starts
+        const bool last = share + 1 == shares;
+        if (__syncthreads_or(last && acc != __ldg(chunk_hist + ((size_t)b * kEncChunks + cA) * 256 + t))) {
+            if (t == 0) S.bad = 1;
+        }
         __syncthreads();
     }
+    // every node's cursor ends exactly at the end of its body (where the
+    // item is the block's last)
+    const bool ends = whole || (cA + 1 == nw && share + 1 == shares);
+    const bool bad = __syncthreads_or(S.bad || (ends && t < V && S.pos[t] != S.end[t]));
     if (t == 0) {
-        // every node's cursor ends exactly at the end of its bitmap (of the
-        // item's part of it)
-        uint32_t bad = S.bad;
-        for (int v = 0; v < V && !bad; v++) bad = S.pos[v] != S.bitsrc[v] + S.nv[v];
         if (whole) {
             status[b] = bad ? PIVCO_ERR_INVALID_ARG : PIVCO_OK;
             rec_bytes[b] = bad ? 0 : rec_bound;
@@ -868,35 +904,38 @@ __global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm) encode_kernel(cons
     extern __shared__ __align__(128) uint8_t smem_raw[];
     EncSmem &S = *reinterpret_cast<EncSmem *>(smem_raw);
     if (chunk_hist && layout_of(layout, (int)blockIdx.x)->big) return;
-    encode_item<true, EncSmem>((int)blockIdx.x, 0, kEncChunks, in, blk_off, layout, chunk_hist, out, out_off,
-                               rec_bytes, status, S);
+    encode_item<true>((int)blockIdx.x, 0, 0, 1, in, blk_off, layout, chunk_hist, out, out_off, rec_bytes, status, S);
 }
 
-// The work list of big blocks' chunks, (block, chunk) by (block, chunk):
-// persistent CTAs take tickets until the list is done.
-__global__ void __launch_bounds__(kEncThreads, kEncChunkCtasPerSm) encode_chunks_kernel(const uint8_t *__restrict__ in,
-                                                                                   const uint64_t *__restrict__ blk_off,
-                                                                                   BlockLayout *__restrict__ layout,
-                                                                                   const uint32_t *__restrict__ chunk_hist,
-                                                                                   uint8_t *__restrict__ out,
-                                                                                   const uint64_t *__restrict__ out_off,
-                                                                                   uint64_t *__restrict__ rec_bytes,
-                                                                                   int32_t *__restrict__ status) {
+// The work list of big blocks' chunks, (block, chunk) by (block, chunk), or
+// by shares of a chunk when the chunks alone would leave CTAs without work (a
+// share counts the chunk's symbols before it again, so only then): persistent
+// CTAs take tickets until the list is done.
+__global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm) encode_chunks_kernel(const uint8_t *__restrict__ in,
+                                                                              const uint64_t *__restrict__ blk_off,
+                                                                              BlockLayout *__restrict__ layout,
+                                                                              const uint32_t *__restrict__ chunk_hist,
+                                                                              uint8_t *__restrict__ out,
+                                                                              const uint64_t *__restrict__ out_off,
+                                                                              uint64_t *__restrict__ rec_bytes,
+                                                                              int32_t *__restrict__ status) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
-    EncSmemBig &S = *reinterpret_cast<EncSmemBig *>(smem_raw);
+    EncSmem &S = *reinterpret_cast<EncSmem *>(smem_raw);
     __shared__ uint32_t s_tk;
-    const uint32_t items = *reinterpret_cast<volatile uint32_t *>(&layout->list_len) * kEncChunks;
+    const uint32_t chunks = *reinterpret_cast<volatile uint32_t *>(&layout->list_len) * kEncChunks;
+    if (chunks == 0) return;
+    const uint32_t shares = min(kEncShares, max(1u, gridDim.x / chunks)), items = chunks * shares;
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) s_tk = atomicAdd(&layout->list_ticket, 1u);
         __syncthreads();
         const uint32_t tk = s_tk;
         if (tk >= items) return;
-        const int bb = (int)layout_of(layout, (int)(tk / kEncChunks))->list_entry;
-        const uint32_t c = tk % kEncChunks;
+        const int bb = (int)layout_of(layout, (int)(tk / (kEncChunks * shares)))->list_entry;
+        const uint32_t c = tk / shares % kEncChunks;
         if (c < enc_nchunks(blk_off[bb + 1] - blk_off[bb]))
-            encode_item<false, EncSmemBig>(bb, c, c + 1, in, blk_off, layout, chunk_hist, out, out_off, rec_bytes,
-                                           status, S);
+            encode_item<false>(bb, c, tk % shares, shares, in, blk_off, layout, chunk_hist, out, out_off, rec_bytes,
+                               status, S);
     }
 }
 
@@ -917,13 +956,13 @@ cudaError_t launch_encode(const uint8_t *in, const uint64_t *blk_off, int nblk, 
     encode_kernel<<<nblk, kEncThreads, smem, st>>>(in, blk_off, layout, chunk_hist, out, out_off, rec_bytes, status);
     count_launches(1);
     if (chunk_hist) {
-        const int smem_big = (int)sizeof(EncSmemBig);
+        const int smem_big = (int)sizeof(EncSmem);
         e = cudaFuncSetAttribute(encode_chunks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_big);
         if (e != cudaSuccess) return e;
         int dev = 0, sms = 148;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        encode_chunks_kernel<<<sms * kEncChunkCtasPerSm, kEncThreads, smem_big, st>>>(in, blk_off, layout, chunk_hist,
+        encode_chunks_kernel<<<sms * kEncCtasPerSm, kEncThreads, smem_big, st>>>(in, blk_off, layout, chunk_hist,
                                                                                       out, out_off, rec_bytes, status);
         count_launches(1);
     }
@@ -936,7 +975,7 @@ namespace pv {
 cudaError_t prepare_encode_kernels() {
     cudaError_t e = cudaFuncSetAttribute(encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EncSmem));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(encode_chunks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EncSmemBig));
+        e = cudaFuncSetAttribute(encode_chunks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EncSmem));
     return e;
 }
 }  // namespace pv

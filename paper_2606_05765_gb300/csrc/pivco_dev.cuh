@@ -75,7 +75,9 @@ struct BlockLayout {
     uint8_t flat;          // regrouped tree with flat subtrees (record tag PVC2)
     uint8_t depth_first[17];   // first node id at depth d (breadth-first); [d+1]-[d] = count
     uint8_t big;               // the levels of the whole block do not fit the encoder's buffers
-    uint8_t pad1[14];
+    uint8_t pad1[2];
+    uint32_t part;             // symbols of an encoder part whose levels fit its buffers with room to spare
+    uint8_t pad4b[8];
     uint16_t tree_a[17];       // leaf-covered prefix count at depth d (TreeShape::a)
     uint16_t pad2[15];
     uint16_t code[256];    // code of symbol s (lens[s] bits, MSB = first decision; canonical or regrouped)
@@ -427,7 +429,12 @@ inline int div_up(long long a, long long b) { return (int)((a + b - 1) / b); }
 // floor(n w / nw) rounded down to a multiple of 32.  The encoder gives chunk w
 // to its warp w; the chunked histogram counts each chunk on its own.
 constexpr uint32_t kEncChunks = 8;
-constexpr int kEBuf = 13824;         // symbols per encoder level buffer (a skew80 64 KiB block in one chunk)
+constexpr int kEBuf = 22016;         // symbols per encoder level buffer (4 CTAs per SM)
+constexpr uint32_t kEncShares = 8;   // shares of a chunk at most
+// Batches of at most this many blocks split their blocks of at least this
+// size over several CTAs (26 blocks of 39-79 KB: FEW_OLD us by one CTA each,
+// FEW_NEW us by chunks)
+constexpr uint32_t kEncFewBlocks = 152, kEncFewSize = 16384;
 constexpr uint32_t kEncMinChunk = 4096;
 __host__ __device__ inline uint32_t enc_nchunks(uint64_t n) {
     const uint64_t c = n / kEncMinChunk;
