@@ -432,8 +432,8 @@ constexpr uint32_t kEncChunks = 8;
 constexpr int kEBuf = 22016;         // symbols per encoder level buffer (4 CTAs per SM)
 constexpr uint32_t kEncShares = 8;   // shares of a chunk at most
 // Batches of at most this many blocks split their blocks of at least this
-// size over several CTAs (26 blocks of 39-79 KB: FEW_OLD us by one CTA each,
-// FEW_NEW us by chunks)
+// size over several CTAs (26 blocks of 39-79 KB: 162 us by one CTA each,
+// 124 us by chunks)
 constexpr uint32_t kEncFewBlocks = 152, kEncFewSize = 16384;
 constexpr uint32_t kEncMinChunk = 4096;
 __host__ __device__ inline uint32_t enc_nchunks(uint64_t n) {
