@@ -9,82 +9,50 @@ namespace pv {
 
 // ---------------------------------------------------------------------------
 // Histogram.  Grid (nblk, slices); each CTA counts one slice of one block.
-// Per-warp shared histograms.  Skewed data (P(top) up to 0.95) would
-// serialise on the most frequent byte's counter, so each warp samples its
-// most frequent byte and counts it in 32 per-lane counters (bins 256 + lane,
-// one bank each), summed into its bin at the end; every byte is one
-// shared-memory add, with no branch.
+// Per-warp shared histograms, one shared-memory add per byte.  What bounds it:
+// instruction issue (three a byte) and shared-memory wavefronts.  Equal bytes
+// of a warp's add do not serialise here: giving the most frequent byte a
+// counter per lane took 86 us for 4096 blocks of 64 KiB of 80 % one byte,
+// leaving it out by a predicate 121 us, adding every byte as it is 60 us.
 // ---------------------------------------------------------------------------
 constexpr int kHistThreads = 256;
 constexpr int kHistWarps = kHistThreads / 32;
-constexpr int kHistBins = 256 + 32;
+constexpr int kHistBins = 256;
 
 __global__ void zero_u32_kernel(uint32_t *p, size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) p[i] = 0;
 }
 
-// counts byte v: the hot byte in the lane's own counter
-__device__ inline void hist_add_byte(uint32_t v, uint32_t hot, uint32_t hot_bin, uint32_t *wh) {
-    atomicAdd(&wh[v == hot ? hot_bin : v], 1u);
-}
-__device__ inline void hist_add_word(uint32_t w, uint32_t hot, uint32_t hot_bin, uint32_t *wh) {
+__device__ inline void hist_add_vec(const uint4 &q, uint32_t *wh) {
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-    for (int k = 0; k < 4; k++) hist_add_byte(__byte_perm(w, 0u, 0x4440u + k), hot, hot_bin, wh);
-}
-__device__ inline void hist_add_vec(const uint4 &q, uint32_t hot, uint32_t hot_bin, uint32_t *wh) {
-    hist_add_word(q.x, hot, hot_bin, wh);
-    hist_add_word(q.y, hot, hot_bin, wh);
-    hist_add_word(q.z, hot, hot_bin, wh);
-    hist_add_word(q.w, hot, hot_bin, wh);
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int k = 0; k < 4; k++) atomicAdd(&wh[__byte_perm(w[i], 0u, 0x4440u + k)], 1u);
 }
 
-// The most frequent of 32 samples of in[lo, hi) (warp-uniform; 0 when empty)
-__device__ inline uint32_t hist_hot_byte(const uint8_t *__restrict__ in, uint64_t lo, uint64_t hi) {
-    const int lane = threadIdx.x & 31;
-    if (hi <= lo) return 0;
-    const uint64_t pos = lo + ((uint64_t)lane * 2654435761u) % (hi - lo);
-    const uint32_t v = in[pos];
-    const uint32_t peers = __match_any_sync(0xffffffffu, v);
-    int best = __popc(peers), bl = lane;
-    for (int o = 16; o; o >>= 1) {
-        const int ob = __shfl_xor_sync(0xffffffffu, best, o), ol = __shfl_xor_sync(0xffffffffu, bl, o);
-        if (ob > best || (ob == best && ol < bl)) { best = ob; bl = ol; }
-    }
-    return __shfl_sync(0xffffffffu, v, bl);
-}
-
-// Counts in[lo, hi) into the warp's histogram my (kHistBins, zeroed) with
-// stride-`step` work sharing starting at `first` (lane or thread index):
-// head bytes up to 16-byte alignment, 16-byte loads four in flight, the tail.
+// Counts in[lo, hi) into the warp's histogram my (zeroed) with stride-`step`
+// work sharing starting at `first` (lane or thread index): head bytes up to
+// 16-byte alignment, 16-byte loads four in flight, the tail.
 __device__ inline void hist_range(const uint8_t *__restrict__ in, uint64_t lo, uint64_t hi, uint32_t first,
-                                  uint32_t step, uint32_t hot, uint32_t *my) {
-    const uint32_t hot_bin = 256u + (threadIdx.x & 31);
+                                  uint32_t step, uint32_t *my) {
     // (the 16-byte boundary of the address: `in` itself may be unaligned)
     uint64_t a = lo + ((16u - (uint32_t)(reinterpret_cast<uintptr_t>(in + lo) & 15u)) & 15u);
     if (a > hi) a = hi;
-    for (uint64_t i = lo + first; i < a; i += step) hist_add_byte(in[i], hot, hot_bin, my);
+    if (lo + first < a) atomicAdd(&my[in[lo + first]], 1u);
     const uint64_t nvec = (hi - a) / 16;
-    const uint4 *vp = reinterpret_cast<const uint4 *>(in + a);
+    const uint4 *vp = reinterpret_cast<const uint4 *>(in + a) + first;
     uint64_t i = first;
-    for (; i + 3 * step < nvec; i += 4 * step) {
+    for (; i + 3 * step < nvec; i += 4 * step, vp += 4 * step) {
         uint4 q[4];
 #pragma unroll
-        for (int u = 0; u < 4; u++) q[u] = __ldg(vp + i + u * step);
+        for (int u = 0; u < 4; u++) q[u] = __ldg(vp + u * step);
 #pragma unroll
-        for (int u = 0; u < 4; u++) hist_add_vec(q[u], hot, hot_bin, my);
+        for (int u = 0; u < 4; u++) hist_add_vec(q[u], my);
     }
-    for (; i < nvec; i += step) hist_add_vec(__ldg(vp + i), hot, hot_bin, my);
-    for (uint64_t j = a + nvec * 16 + first; j < hi; j += step) hist_add_byte(in[j], hot, hot_bin, my);
-}
-
-// Adds the warp's 32 hot-byte counters into the hot byte's bin (whole warp,
-// after its counting)
-__device__ inline void hist_fold_hot(uint32_t *my, uint32_t hot) {
-    const int lane = threadIdx.x & 31;
-    __syncwarp();
-    const uint32_t c = __reduce_add_sync(0xffffffffu, my[256 + lane]);
-    if (lane == 0) my[hot] += c;
-    __syncwarp();
+    for (; i < nvec; i += step, vp += step) hist_add_vec(__ldg(vp), my);
+    const uint64_t j = a + nvec * 16 + first;
+    if (j < hi) atomicAdd(&my[in[j]], 1u);
 }
 
 __global__ void __launch_bounds__(kHistThreads) histogram_kernel(const uint8_t *__restrict__ in,
@@ -98,10 +66,8 @@ __global__ void __launch_bounds__(kHistThreads) histogram_kernel(const uint8_t *
     const uint64_t span = ((n + slices - 1) / slices + 15) & ~uint64_t(15);
     const uint64_t lo = lo0 + min(n, span * sl), hi = lo0 + min(n, span * (sl + 1));
     for (int i = t; i < kHistWarps * kHistBins; i += kHistThreads) (&wh[0][0])[i] = 0;
-    const uint32_t hot = hist_hot_byte(in, lo, hi);
     __syncthreads();
-    hist_range(in, lo, hi, (uint32_t)t, kHistThreads, hot, wh[warp]);
-    hist_fold_hot(wh[warp], hot);
+    hist_range(in, lo, hi, (uint32_t)t, kHistThreads, wh[warp]);
     __syncthreads();
     for (int s = t; s < 256; s += kHistThreads) {
         uint32_t sum = 0;
@@ -142,10 +108,8 @@ __device__ inline void histogram_chunks_block(int b, const uint8_t *__restrict__
     const uint64_t lo = blk_off[b] + enc_chunk_start(n, warp, nw), hi = blk_off[b] + enc_chunk_start(n, warp + 1, nw);
     uint32_t *my = wh[warp];
     for (int i = lane; i < kHistBins; i += 32) my[i] = 0;
-    const uint32_t hot = hist_hot_byte(in, lo, hi);
     __syncwarp();
-    hist_range(in, lo, hi, (uint32_t)lane, 32u, hot, my);
-    hist_fold_hot(my, hot);
+    hist_range(in, lo, hi, (uint32_t)lane, 32u, my);
     __syncthreads();
     for (int s = t; s < 256; s += kHistThreads) {
         uint32_t sum = 0;
@@ -157,6 +121,25 @@ __device__ inline void histogram_chunks_block(int b, const uint8_t *__restrict__
         hist[(size_t)b * 256 + s] = sum;
         if (h_sm) h_sm[s] = sum;
     }
+}
+
+// Chunk c of block b by one CTA (256 threads).
+__device__ inline void histogram_one_chunk(int b, uint32_t c, const uint8_t *__restrict__ in,
+                                           const uint64_t *__restrict__ blk_off, uint32_t *__restrict__ chunk_hist,
+                                           uint32_t (*wh)[kHistBins]) {
+    const int t = threadIdx.x, warp = t >> 5;
+    const uint64_t n = blk_off[b + 1] - blk_off[b];
+    const uint32_t nw = enc_nchunks(n);
+    const uint64_t lo = blk_off[b] + enc_chunk_start(n, c, nw), hi = blk_off[b] + enc_chunk_start(n, c + 1, nw);
+#pragma unroll
+    for (int w = 0; w < kHistWarps; w++) wh[w][t] = 0;
+    __syncthreads();
+    hist_range(in, lo, hi, (uint32_t)t, kHistThreads, wh[warp]);
+    __syncthreads();
+    uint32_t sum = 0;
+#pragma unroll
+    for (int w = 0; w < kHistWarps; w++) sum += wh[w][t];
+    chunk_hist[((size_t)b * kEncChunks + c) * 256 + t] = sum;
 }
 
 __global__ void __launch_bounds__(kHistThreads) histogram_chunks_kernel(const uint8_t *__restrict__ in,
@@ -186,52 +169,72 @@ cudaError_t launch_histogram_chunks(const uint8_t *in, const uint64_t *blk_off, 
 // and following packages down: at each level the selected items are a
 // prefix of the list; its leaves are the lightest leaves, and each gains one
 // bit of length; its packages select twice as many items one level deeper.
+// What bounds it: instruction issue with many blocks, the chain of levels with
+// few.  (With 64-bit sort keys, every symbol sorted, and the two searches of a
+// level one after the other, the step took 2350 instructions a warp, 77 us for
+// 4096 blocks of 256 symbols; now 2010 and 65 us.  Each level as one merge by
+// 64 threads took fewer, but its longer chain made it 84 us.)
 // ---------------------------------------------------------------------------
 constexpr int kPmThreads = 256;
 
-// # of a[0..256) below x, a sorted with its unused tail holding the type's
-// maximum (above every x searched for): binary lifting over 255 places, then
-// one compare for the last, with no bounds checks
-template <typename W>
-__device__ inline int count_less_w(const W *a, W x) {
-    int pos = 0;
-#pragma unroll
-    for (int step = 128; step >= 1; step >>= 1) pos = a[pos + step - 1] < x ? pos + step : pos;
-    return pos + (a[pos] < x ? 1 : 0);
+__device__ inline uint32_t pm_lds(uint32_t at, uint32_t) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+    return v;
 }
-// # of a[0..256) not above x (the same tail)
+__device__ inline uint64_t pm_lds(uint32_t at, uint64_t) {
+    uint64_t v;
+    asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(at) : "memory");
+    return v;
+}
+
+// less: # of a[0..256) below x; le: # of b[0..256) not above y.  a and b are
+// sorted, their unused tails holding the type's maximum (above every x and y
+// searched for): binary lifting over 255 places, then one compare for the
+// last, with no bounds checks; the two chains side by side, a load, a compare
+// and an add a step each.
 template <typename W>
-__device__ inline int count_le_w(const W *a, W x) {
-    int pos = 0;
+__device__ inline void pm_search(const W *a, W x, const W *b, W y, int &less, int &le) {
+    constexpr uint32_t z = sizeof(W);
+    const uint32_t a0 = (uint32_t)__cvta_generic_to_shared(a), b0 = (uint32_t)__cvta_generic_to_shared(b);
+    uint32_t pa = a0, pb = b0;
 #pragma unroll
-    for (int step = 128; step >= 1; step >>= 1) pos = a[pos + step - 1] <= x ? pos + step : pos;
-    return pos + (a[pos] <= x ? 1 : 0);
+    for (uint32_t step = 128; step >= 1; step >>= 1) {
+        const W va = pm_lds(pa + (step - 1) * z, W(0)), vb = pm_lds(pb + (step - 1) * z, W(0));
+        pa += va < x ? step * z : 0u;
+        pb += vb <= y ? step * z : 0u;
+    }
+    const W va = pm_lds(pa, W(0)), vb = pm_lds(pb, W(0));
+    less = (int)((pa - a0) / z) + (va < x ? 1 : 0);
+    le = (int)((pb - b0) / z) + (vb <= y ? 1 : 0);
 }
 
 // Levels max_len - 1 .. 1 of package-merge: each level merges the sorted
 // leaves with the packages of the level below; leafpos[l][i] is leaf i's
-// place at level l.  W: the weight type (32 bits when no package can reach
-// 2^32 - 1, which halves the shared-memory traffic of the searches).  leafw
+// position at level l.  W is wide enough for every weight.  leafw[0..256)
 // (256 places) holds the type's maximum past the K leaves; pw is given the
 // same tail at every level, so the searches need no bounds.
 template <typename W>
 __device__ inline void pm_levels(const W *leafw, W *pw, W (*lw)[512], uint16_t (*leafpos)[256], int K, int max_len) {
     const int t = threadIdx.x;
-    for (int i = t; i < K; i += kPmThreads) { lw[max_len & 1][i] = leafw[i]; leafpos[max_len][i] = (uint16_t)i; }
+    const bool on = (t & ~31) < K;   // (a level has no more packages than leaves)
+    const W x = leafw[t];
+    if (t < K) lw[max_len & 1][t] = x;
     int len_prev = K;
     __syncthreads();
     for (int lvl = max_len - 1; lvl >= 1; lvl--) {
         const W *prev = lw[(lvl + 1) & 1];
         W *cur = lw[lvl & 1];
         const int P = len_prev / 2;
-        for (int j = t; j < 256; j += kPmThreads) pw[j] = j < P ? prev[2 * j] + prev[2 * j + 1] : ~W(0);
+        const W y = t < P ? prev[2 * t] + prev[2 * t + 1] : ~W(0);
+        pw[t] = y;
         __syncthreads();
-        for (int i = t; i < K; i += kPmThreads) {
-            const int pos = i + count_less_w(pw, leafw[i]);
-            cur[pos] = leafw[i];
-            leafpos[lvl][i] = (uint16_t)pos;
+        if (on) {
+            int less, le;
+            pm_search<W>(pw, x, leafw, y, less, le);
+            if (t < K) { cur[t + less] = x; leafpos[lvl][t] = (uint16_t)(t + less); }
+            if (t < P) cur[t + le] = y;
         }
-        for (int j = t; j < P; j += kPmThreads) cur[j + count_le_w(leafw, pw[j])] = pw[j];
         len_prev = K + P;
         __syncthreads();
     }
@@ -244,57 +247,86 @@ struct ClSmem {
     uint64_t pw[256];
     uint16_t leafpos[kMaxLen + 1][256];
     int32_t s_len[kMaxLen + 2];
+    int32_t wcnt[kPmThreads / 32];
 };
+
+// keys[0 .. N) (N a power of two, 32 .. 256; one key per thread, in key) sorted
+// ascending by a bitonic network; steps within a warp exchange by shuffle, the
+// others through x (two buffers in turn).  Whole CTA.
+template <typename T>
+__device__ inline T pm_sort(T key, int N, T (*x)[256]) {
+    const int t = threadIdx.x;
+    int flip = 0;
+#pragma unroll
+    for (int k = 2; k <= 256; k <<= 1) {
+        if (k > N) break;
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            T other = key;
+            if (j >= 32) {
+                x[flip][t] = key;
+                __syncthreads();
+                other = x[flip][t ^ j];
+                flip ^= 1;
+            } else {
+                other = __shfl_xor_sync(0xffffffffu, key, j);
+            }
+            // the lower partner keeps the smaller key in an ascending run
+            key = ((t & j) == 0) == ((t & k) == 0) ? min(key, other) : max(key, other);
+        }
+    }
+    return key;
+}
 
 // Code lengths of the histogram h (shared, 256) into lens (shared, 256) by
 // one CTA of 256 threads; returns the status (every thread).
 __device__ inline int code_lengths_block(const uint32_t *h, int max_len, ClSmem &C, uint8_t *lens) {
-    uint64_t *leafw = C.leafw, *pw = C.pw;
     uint8_t *leafsym = C.leafsym;
-    uint64_t (*lw)[512] = C.lw;
-    uint16_t (*leafpos)[256] = C.leafpos;
     int32_t *s_len = C.s_len;
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     lens[t] = 0;
-    const int K = __syncthreads_count(h[t] != 0);
+    const uint32_t cnt = h[t];
+    const uint32_t pm = __ballot_sync(0xffffffffu, cnt != 0);
+    if (lane == 0) C.wcnt[warp] = __popc(pm);
+    const bool wide = __syncthreads_or(cnt >= 0xFFFFFFu);   // (a count that needs a 64-bit key)
+    int K = 0, before = 0;
+#pragma unroll
+    for (int w = 0; w < kPmThreads / 32; w++) {
+        if (w == warp) before = K;
+        K += C.wcnt[w];
+    }
     if (K >= 2 && K <= (1 << max_len)) {
-        // present symbols sorted by (count, symbol): bitonic sort of one key per
-        // thread (absent symbols sort last); in-warp steps exchange by shuffle
-        {
-            uint64_t key = h[t] ? (((uint64_t)h[t] << 8) | (uint64_t)t) : ~0ull;
-            for (int k = 2; k <= 256; k <<= 1) {
-                for (int j = k >> 1; j > 0; j >>= 1) {
-                    uint64_t other;
-                    if (j >= 32) {
-                        pw[t] = key;
-                        __syncthreads();
-                        other = pw[t ^ j];
-                        __syncthreads();
-                    } else {
-                        other = __shfl_xor_sync(0xffffffffu, key, j);
-                    }
-                    const bool lower = (t & j) == 0, up = (t & k) == 0;
-                    // the lower partner keeps the smaller key in an ascending run
-                    key = (lower == up) ? (key < other ? key : other) : (key < other ? other : key);
-                }
-            }
-            leafw[t] = t < K ? key >> 8 : ~0ull;   // (the searches' tail past the leaves)
-            if (t < K) leafsym[t] = (uint8_t)(key & 0xFF);
+        // present symbols sorted by (count, symbol)
+        int N = 32;
+        while (N < K) N <<= 1;
+        const int at = before + __popc(pm & ((1u << lane) - 1u));
+        uint64_t w = ~0ull;
+        if (!wide) {
+            uint32_t (*x)[256] = reinterpret_cast<uint32_t (*)[256]>(&C.lw[0][0]);   // (two buffers, then the keys)
+            if (cnt) x[2][at] = (cnt << 8) | (uint32_t)t;
+            __syncthreads();
+            const uint32_t key = pm_sort<uint32_t>(t < K ? x[2][t] : 0xFFFFFFFFu, N, x);
+            if (t < K) { w = key >> 8; leafsym[t] = (uint8_t)key; }
+        } else {
+            uint64_t (*x)[256] = reinterpret_cast<uint64_t (*)[256]>(&C.lw[0][0]);
+            if (cnt) x[2][at] = ((uint64_t)cnt << 8) | (uint64_t)t;
+            __syncthreads();
+            const uint64_t key = pm_sort<uint64_t>(t < K ? x[2][t] : ~0ull, N, x);
+            if (t < K) { w = key >> 8; leafsym[t] = (uint8_t)key; }
         }
-        __syncthreads();
         // an item of a level holds at most one copy of a leaf per level
         // below, so no weight exceeds max_len * K * (largest count); 32-bit
         // weights stay below 2^32 - 1, the searches' tail value
-        if ((uint64_t)max_len * (uint64_t)K * leafw[K - 1] < (1ull << 32) - 1) {
-            uint32_t *leafw32 = reinterpret_cast<uint32_t *>(pw), *pw32 = leafw32 + 256;
-            uint32_t (*lw32)[512] = reinterpret_cast<uint32_t (*)[512]>(&lw[0][0]);
-            const uint32_t w = t < K ? (uint32_t)leafw[t] : 0xFFFFFFFFu;
+        const uint64_t most = t < K ? (uint64_t)max_len * (uint64_t)K * w : 0;
+        if (__syncthreads_or(most >= (1ull << 32) - 1)) {
+            C.leafw[t] = w;     // (the searches' tail past the leaves)
             __syncthreads();
-            leafw32[t] = w;
-            __syncthreads();
-            pm_levels<uint32_t>(leafw32, pw32, lw32, leafpos, K, max_len);
+            pm_levels<uint64_t>(C.leafw, C.pw, C.lw, C.leafpos, K, max_len);
         } else {
-            pm_levels<uint64_t>(leafw, pw, lw, leafpos, K, max_len);
+            uint32_t *leafw32 = reinterpret_cast<uint32_t *>(C.pw), *pw32 = leafw32 + 256;
+            leafw32[t] = (uint32_t)w;
+            __syncthreads();
+            pm_levels<uint32_t>(leafw32, pw32, reinterpret_cast<uint32_t (*)[512]>(&C.lw[0][0]), C.leafpos, K, max_len);
         }
         // selection, top-down (one warp): at each level the selected items are
         // the first m; count the leaves among them (their positions increase
@@ -303,13 +335,13 @@ __device__ inline int code_lengths_block(const uint32_t *h, int max_len, ClSmem 
             int m = 2 * K - 2;
             for (int lvl = 1; lvl <= max_len; lvl++) {
                 const int last = min(8 * t + 7, K - 1);
-                const bool full = 8 * t < K && leafpos[lvl][last] < m;
+                const bool full = 8 * t < K && (lvl < max_len ? (int)C.leafpos[lvl][last] : last) < m;
                 const int nb = __popc(__ballot_sync(0xffffffffu, full));
                 const int i2 = 8 * nb + t;
-                const bool below = t < 8 && i2 < K && leafpos[lvl][min(i2, 255)] < m;
-                const int cnt = min(8 * nb, K) + __popc(__ballot_sync(0xffffffffu, below));
-                if (t == 0) s_len[lvl] = cnt;
-                m = 2 * (m - cnt);
+                const bool below = t < 8 && i2 < K && (lvl < max_len ? (int)C.leafpos[lvl][min(i2, 255)] : i2) < m;
+                const int c = min(8 * nb, K) + __popc(__ballot_sync(0xffffffffu, below));
+                if (t == 0) s_len[lvl] = c;
+                m = 2 * (m - c);
             }
         }
         __syncthreads();
@@ -383,11 +415,12 @@ struct LaySmem {
     TreeShape ts;
     FlatTree F;
     unsigned long long s_part[kLayThreads / 32];
+    float s_partf[kLayThreads / 32];
 };
 
 // Layout of block b from its histogram h and lengths lens (both shared, 256)
 // by one CTA of 256 threads: written to layout[b], rec_bound[b], status[b].
-__device__ inline void build_layout_block(int b, const uint32_t *h, const uint8_t *lens, const SelectParams &sp,
+__device__ inline void build_layout_block(int b, int nblk, const uint32_t *h, const uint8_t *lens, const SelectParams &sp,
                                           LaySmem &Y, BlockLayout *__restrict__ layout,
                                           uint64_t *__restrict__ rec_bound, int32_t *__restrict__ status) {
     BlockLayout &L = Y.L;
@@ -440,8 +473,10 @@ __device__ inline void build_layout_block(int b, const uint32_t *h, const uint8_
                 L.flat = flat ? 1 : 0;
                 L.n_int = (uint16_t)V;
                 L.max_depth = (uint8_t)maxd;
-                for (int d = 0; d <= 16; d++) L.depth_first[d] = (uint8_t)(d < maxd ? fst[d] : V);
-                for (int d = 0; d <= 16; d++) L.tree_a[d] = (uint16_t)(flat ? F.a[d] : ts.a[d]);
+            }
+            if (t <= 16) {
+                L.depth_first[t] = (uint8_t)(t < maxd ? fst[t] : V);
+                L.tree_a[t] = (uint16_t)(flat ? F.a[t] : ts.a[t]);
             }
             if (flat) {
                 // regrouped codes (symbol x of item i is (code_i << D) | x) and
@@ -545,27 +580,28 @@ __device__ inline void build_layout_block(int b, const uint32_t *h, const uint8_
                 // encoder level buffer (spans of whole 16-byte units), or
                 // the batch has too few blocks to fill the chip with one CTA
                 // each
-                if (t == 0 && gridDim.x <= kEncFewBlocks && n >= kEncFewSize && maxd > 1) L.big = 1;
-                unsigned long long part = n;
-                if (t >= 1 && t < maxd) {
-                    uint64_t lvl = 0, raw = 0;
-                    for (int v = fst[t]; v < fst[t + 1]; v++) {
-                        lvl += ((uint64_t)L.nv[v] + 15u) & ~15ull;
+                if (t == 0 && nblk <= (int)kEncFewBlocks && n >= kEncFewSize && maxd > 1) L.big = 1;
+                float part = (float)n;   // (1024 symbols and more: its rounding is far below the 10 % to spare)
+                for (int d = 1 + (t >> 5); d < maxd; d += kLayThreads / 32) {   // a warp per level
+                    uint32_t raw = 0, pad = 0;
+                    for (int v = fst[d] + (t & 31); v < fst[d + 1]; v += 32) {
                         raw += L.nv[v];
+                        pad += (0u - L.nv[v]) & 15u;
                     }
-                    if (lvl > (uint64_t)kEBuf && enc_nchunks(n) >= 2) L.big = 1;
+                    raw = __reduce_add_sync(0xffffffffu, raw);
+                    pad = __reduce_add_sync(0xffffffffu, pad);
+                    if ((t & 31) == 0 && (uint64_t)raw + pad > (uint64_t)kEBuf && enc_nchunks(n) >= 2) L.big = 1;
                     // a part's level: its share of the level and the spans' rounding, 10 % to spare
-                    const uint64_t room = (uint64_t)kEBuf - 16ull * (uint32_t)(fst[t + 1] - fst[t]);
-                    if (raw) part = room * n / raw / 10 * 9;
+                    const float room = 0.9f * (float)(kEBuf - 16 * (fst[d + 1] - fst[d]));
+                    if (raw) part = fminf(part, room * (float)n / (float)raw);
                 }
-                if (t < 32) {
-#pragma unroll
-                    for (int o = 16; o; o >>= 1) {
-                        const unsigned long long y = __shfl_xor_sync(0xffffffffu, part, o);
-                        part = y < part ? y : part;
-                    }
+                if ((t & 31) == 0) Y.s_partf[t >> 5] = part;
+                __syncthreads();
+                if (t == 0) {
+                    for (int w = 1; w < kLayThreads / 32; w++) part = fminf(part, Y.s_partf[w]);
+                    const uint32_t p = (uint32_t)min((unsigned long long)part, (unsigned long long)n);
                     // (in whole rounds of the encoder's eight windows, where it holds one)
-                    if (t == 0) L.part = (uint32_t)(part >= 8192 ? part & ~8191ull : part & ~1023ull);
+                    L.part = p >= 8192 ? p & ~8191u : p & ~1023u;
                 }
                 __syncthreads();
             if (t < 32) {
@@ -628,7 +664,7 @@ __global__ void __launch_bounds__(kLayThreads) build_layout_kernel(const uint32_
     const int b = blockIdx.x, t = threadIdx.x;
     h[t] = hist[(size_t)b * 256 + t];
     lens[t] = lens_in[(size_t)b * 256 + t];
-    build_layout_block(b, h, lens, sp, Y, layout, rec_bound, status);
+    build_layout_block(b, gridDim.x, h, lens, sp, Y, layout, rec_bound, status);
 }
 
 // The encoder's planning in one launch, one CTA per block: chunk histograms,
@@ -644,24 +680,59 @@ struct PlanSmem {
     } u;
 };
 
-__global__ void __launch_bounds__(kHistThreads) block_plan_kernel(const uint8_t *__restrict__ in,
-                                                                  const uint64_t *__restrict__ blk_off, int max_len,
-                                                                  const __grid_constant__ SelectParams sp,
-                                                                  uint32_t *__restrict__ hist,
-                                                                  uint32_t *__restrict__ chunk_hist,
-                                                                  uint8_t *__restrict__ lens_out,
-                                                                  BlockLayout *__restrict__ layout,
-                                                                  uint64_t *__restrict__ rec_bound,
-                                                                  int32_t *__restrict__ status) {
-    static_assert(kHistThreads == kPmThreads && kPmThreads == kLayThreads, "one CTA shape for the three steps");
-    __shared__ PlanSmem P;
-    const int b = blockIdx.x, t = threadIdx.x;
-    histogram_chunks_block(b, in, blk_off, hist, chunk_hist, P.u.wh, P.h);
+// Batches of at most one block per SM run as clusters of one CTA per chunk: a
+// block of at least kPlanWide symbols is counted by all eight, a smaller one
+// by the first.  (One block of 1 MiB: 93 us by one CTA, 35 us by eight; 509
+// text-like blocks 57 and 62 us, 1024 mixed blocks 135 and 125 us: with blocks
+// enough for every SM the extra CTAs' coming and going takes what they save.)
+constexpr uint32_t kPlanWide = 32768;
+
+__device__ inline void plan_rest(int b, int nblk, int max_len, const SelectParams &sp, PlanSmem &P,
+                                 uint8_t *__restrict__ lens_out, BlockLayout *__restrict__ layout,
+                                 uint64_t *__restrict__ rec_bound, int32_t *__restrict__ status) {
     __syncthreads();
     code_lengths_block(P.h, max_len, P.u.cl, P.lens);   // (its status is the layout's too)
-    lens_out[(size_t)b * 256 + t] = P.lens[t];
+    lens_out[(size_t)b * 256 + threadIdx.x] = P.lens[threadIdx.x];
     __syncthreads();
-    build_layout_block(b, P.h, P.lens, sp, P.u.lay, layout, rec_bound, status);
+    build_layout_block(b, nblk, P.h, P.lens, sp, P.u.lay, layout, rec_bound, status);
+}
+
+static_assert(kHistThreads == kPmThreads && kPmThreads == kLayThreads, "one CTA shape for the three steps");
+
+__global__ void __launch_bounds__(kHistThreads) block_plan_kernel(
+    const uint8_t *__restrict__ in, const uint64_t *__restrict__ blk_off, int max_len,
+    const __grid_constant__ SelectParams sp, uint32_t *__restrict__ hist, uint32_t *__restrict__ chunk_hist,
+    uint8_t *__restrict__ lens_out, BlockLayout *__restrict__ layout, uint64_t *__restrict__ rec_bound,
+    int32_t *__restrict__ status) {
+    __shared__ PlanSmem P;
+    histogram_chunks_block(blockIdx.x, in, blk_off, hist, chunk_hist, P.u.wh, P.h);
+    plan_rest(blockIdx.x, gridDim.x, max_len, sp, P, lens_out, layout, rec_bound, status);
+}
+
+__global__ void __cluster_dims__(kEncChunks, 1, 1) __launch_bounds__(kHistThreads)
+    block_plan_cluster_kernel(const uint8_t *__restrict__ in, const uint64_t *__restrict__ blk_off, int max_len,
+                              const __grid_constant__ SelectParams sp, uint32_t *__restrict__ hist,
+                              uint32_t *__restrict__ chunk_hist, uint8_t *__restrict__ lens_out,
+                              BlockLayout *__restrict__ layout, uint64_t *__restrict__ rec_bound,
+                              int32_t *__restrict__ status) {
+    __shared__ PlanSmem P;
+    const int b = blockIdx.x / kEncChunks, t = threadIdx.x;
+    const uint32_t c = blockIdx.x % kEncChunks;
+    const uint64_t n = blk_off[b + 1] - blk_off[b];
+    if (n >= kPlanWide) {   // (all CTAs of the cluster take the same way)
+        histogram_one_chunk(b, c, in, blk_off, chunk_hist, P.u.wh);
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (c) return;
+        uint32_t sum = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < kEncChunks; w++) sum += __ldcg(&chunk_hist[((size_t)b * kEncChunks + w) * 256 + t]);
+        hist[(size_t)b * 256 + t] = sum;
+        P.h[t] = sum;
+    } else {
+        if (c) return;
+        histogram_chunks_block(b, in, blk_off, hist, chunk_hist, P.u.wh, P.h);
+    }
+    plan_rest(b, gridDim.x / kEncChunks, max_len, sp, P, lens_out, layout, rec_bound, status);
 }
 
 cudaError_t launch_block_plan(const uint8_t *in, const uint64_t *blk_off, int nblk, const pivco_params &p,
@@ -672,8 +743,15 @@ cudaError_t launch_block_plan(const uint8_t *in, const uint64_t *blk_off, int nb
     sp.p = p;
     const AnsTables &T = host_ans_tables();
     for (int i = 0; i < 50; i++) sp.fseh_q16[i] = T.fseh_q16[i];
-    block_plan_kernel<<<nblk, kHistThreads, 0, st>>>(in, blk_off, p.max_len, sp, hist, chunk_hist, lens, layout,
-                                                     rec_bound, status);
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (nblk <= sms)
+        block_plan_cluster_kernel<<<nblk * (int)kEncChunks, kHistThreads, 0, st>>>(in, blk_off, p.max_len, sp, hist, chunk_hist,
+                                                                                    lens, layout, rec_bound, status);
+    else
+        block_plan_kernel<<<nblk, kHistThreads, 0, st>>>(in, blk_off, p.max_len, sp, hist, chunk_hist, lens, layout,
+                                                         rec_bound, status);
     count_launches(1);
     return cudaGetLastError();
 }

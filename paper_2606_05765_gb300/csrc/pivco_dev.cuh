@@ -149,36 +149,41 @@ __device__ inline void build_tree_shape(const uint8_t *lens, TreeShape &ts, uint
         }
     }
     __syncthreads();
-    if (t == 0) {
-        int32_t a = 0, first = 0, base = 0, K = 0, ml = 0;
-        bool ok = true;
-        ts.a[0] = 0;
-        ts.first[0] = 0;
-        for (int l = 1; l <= (int)kMaxLen; l++) {
-            ts.len_base[l] = base;
-            base += ts.cnt[l];
-            K += ts.cnt[l];
-            if (ts.cnt[l]) ml = l;
+    if (t < 32) {
+        // a lane per depth d: a[d] = sum of cnt[k] 2^(d - k) over k <= d;
+        // open[d] = 2^d - a[d] internal nodes at depth d
+        const uint32_t d = t;
+        const int32_t c = d >= 1 && d <= kMaxLen ? ts.cnt[d] : 0;
+        int32_t a = 0, base = 0, K = 0;
+#pragma unroll
+        for (uint32_t k = 1; k <= kMaxLen; k++) {
+            const int32_t ck = __shfl_sync(0xffffffffu, c, k);
+            if (k <= d) a = 2 * a + ck;
+            if (k < d) base += ck;
+            K += ck;
         }
-        // open[d] = 2^d - a[d] internal nodes at depth d; a[d] = 2 a[d-1] + cnt[d]
-        for (int d = 0; d <= (int)kMaxLen; d++) {
-            if (d > 0) a = 2 * a + ts.cnt[d];
-            ts.a[d] = a;
-            int64_t open = (int64_t(1) << d) - a;
-            if (open < 0) ok = false;
-            ts.first[d] = first;
-            if (d < ml) {
-                if (open <= 0) ok = false;
-                first += (int32_t)open;
-            } else if (d == ml && open != 0) {
-                ok = false;     // Kraft equality: the tree is full
-            }
+        const uint32_t present = __ballot_sync(0xffffffffu, c != 0);
+        const uint32_t ml = present ? 31u - __clz(present) : 0u;
+        const int32_t open = d <= kMaxLen ? (int32_t)(1u << d) - a : 0;
+        // (Kraft equality at the last depth: the tree is full)
+        const bool bad = d <= kMaxLen && (open < 0 || (d < ml && open == 0) || (d == ml && open != 0));
+        const int32_t mine = d < ml ? open : 0;
+        int32_t inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (t >= o) inc += y;
         }
-        ts.first[kMaxLen + 1] = first;
-        ts.n_int = first;
-        ts.max_len = ml;
-        ts.K = K;
-        ts.ok = ok && K >= 2 && first == K - 1;
+        const int32_t total = __shfl_sync(0xffffffffu, inc, 31);
+        const bool ok = !__any_sync(0xffffffffu, bad);
+        if (d <= kMaxLen + 1) { ts.a[d] = a; ts.len_base[d] = base; }
+        if (d <= kMaxLen + 1) ts.first[d] = inc - mine;
+        if (t == 0) {
+            ts.n_int = total;
+            ts.max_len = (int32_t)ml;
+            ts.K = K;
+            ts.ok = ok && K >= 2 && total == K - 1;
+        }
     }
     __syncthreads();
     // rank of s among symbols of the same length (by value): lanes of equal
