@@ -96,11 +96,12 @@ struct BlockLayout {
     uint8_t nhi1[256];
     // scratch of the chunked encoder (the work list of big blocks; written
     // by the encode call, not by the plan): entry i of the list lives in
-    // block i's layout, its length and the chunk ticket in block 0's
+    // block i's layout (with the list's entry that comes i-th by size), its
+    // length and the chunk ticket in block 0's
     uint32_t list_entry;
     uint32_t list_len;
     uint32_t list_ticket;
-    uint32_t pad4;
+    uint32_t list_sorted;
 };
 static_assert(offsetof(BlockLayout, ci) % 16 == 0 && offsetof(BlockLayout, nhi1) + 256 == offsetof(BlockLayout, ci) + 768,
               "the canonical tables are one 16-byte aligned run");
