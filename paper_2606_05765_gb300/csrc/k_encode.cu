@@ -876,16 +876,17 @@ __global__ void __launch_bounds__(kEncThreads) encode_reset_kernel(const uint64_
     else if (L.n != n || (reinterpret_cast<uintptr_t>(rec) & 15)) st = PIVCO_ERR_INVALID_ARG;
     else if (cap < L.rec_bound) st = PIVCO_ERR_CAPACITY;
     if (st != PIVCO_OK) {
-        if (t == 0) { status[b] = st; rec_bytes[b] = 0; }
+        if (t == 0 && blockIdx.y == 0) { status[b] = st; rec_bytes[b] = 0; }
         return;
     }
     // the body and the record's tail, zeroed (the chunks OR their bits in)
     const uint32_t b0 = L.body0, b1 = L.rec_bound;
     const uint32_t h0 = min(b1, (b0 + 15u) & ~15u);
-    for (uint32_t i = b0 + t; i < h0; i += kEncThreads) rec[i] = 0;
-    for (uint32_t i = h0 + 16 * t; i < b1; i += 16 * kEncThreads)
+    const uint32_t tt = blockIdx.y * kEncThreads + t, nt = gridDim.y * kEncThreads;
+    for (uint32_t i = b0 + tt; i < h0; i += nt) rec[i] = 0;
+    for (uint32_t i = h0 + 16 * tt; i < b1; i += 16 * nt)
         *reinterpret_cast<uint4 *>(rec + i) = make_uint4(0u, 0u, 0u, 0u);
-    if (t == 0) {
+    if (tt == 0) {
         status[b] = PIVCO_OK;
         rec_bytes[b] = L.rec_bound;
         const uint32_t i = atomicAdd(&layout->list_len, 1u);
@@ -982,11 +983,17 @@ cudaError_t launch_encode(const uint8_t *in, const uint64_t *blk_off, int nblk, 
     const int smem = (int)sizeof(EncSmem);
     cudaError_t e = cudaFuncSetAttribute(encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // the work list of big blocks: emptied, then filled by the reset pass
     e = cudaMemsetAsync(&layout->list_len, 0, 2 * sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
     if (chunk_hist) {
-        encode_reset_kernel<<<nblk, kEncThreads, 0, st>>>(blk_off, layout, out, out_off, rec_bytes, status);
+        // (several CTAs per block when the blocks alone do not fill the chip: one block of 1 MiB 17 us by one CTA,
+        // 4 by 16; 1024 mixed blocks 31 us by one each, 24 by two)
+        const int per = max(1, min(16, div_up(8 * sms, nblk)));
+        encode_reset_kernel<<<dim3(nblk, per), kEncThreads, 0, st>>>(blk_off, layout, out, out_off, rec_bytes, status);
         count_launches(1);
     }
     encode_kernel<<<nblk, kEncThreads, smem, st>>>(in, blk_off, layout, chunk_hist, out, out_off, rec_bytes, status);
@@ -995,9 +1002,6 @@ cudaError_t launch_encode(const uint8_t *in, const uint64_t *blk_off, int nblk, 
         const int smem_big = (int)sizeof(EncSmem);
         e = cudaFuncSetAttribute(encode_chunks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_big);
         if (e != cudaSuccess) return e;
-        int dev = 0, sms = 148;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         encode_chunks_kernel<<<sms * kEncCtasPerSm, kEncThreads, smem_big, st>>>(in, blk_off, layout, chunk_hist,
                                                                                       out, out_off, rec_bytes, status);
         count_launches(1);
