@@ -61,7 +61,6 @@ struct __align__(16) EncSmem {
     uint32_t lut[256];                      // byte selectors that bring the symbols of a bitmap byte's zeros to the
                                             // front (first four in the low half)
     uint32_t pmask[8];                      // symbols that have a code
-    uint32_t hot;                           // the symbol with the shortest code (the most frequent one)
     uint32_t bad, lvl_max;                  // symbols of the largest level below the root (a part that did not fit)
     uint8_t first[17];
     uint8_t maxd;
@@ -70,7 +69,7 @@ struct __align__(16) EncSmem {
 static_assert(kEncCtasPerSm * (sizeof(EncSmem) + 64 + 1024) <= 228 * 1024, "encoder CTAs per SM");
 static_assert(offsetof(BlockLayout, ci) <= sizeof(EncSmem::buf[1]) && offsetof(BlockLayout, ci) % 16 == 0,
               "the staged part of the layout fits a level buffer");
-static_assert(sizeof(EncSmem::buf[0]) >= 4 * (288 + 256 + 257), "a level buffer holds the counting scratch");
+static_assert(sizeof(EncSmem::buf[0]) >= 4 * (256 + 256 + 257), "a level buffer holds the counting scratch");
 
 template <typename F, typename G>
 __device__ inline uint32_t warp_scan_loop(int n, F f, G out) {
@@ -109,38 +108,6 @@ __device__ inline void ldg32(const uint8_t *p, const uint8_t *end, uint32_t (&x)
         x[j] = sh ? __funnelshift_r(prev, nx, sh) : prev;
         prev = nx;
     }
-}
-
-// adds the 32 bytes x (first vl valid) to a shared histogram of 256 bins
-// and 32 per-lane bins (256 + lane, one bank each) that take the block's most
-// frequent symbol h (skewed data would otherwise serialize on one counter):
-// one shared add per byte, no branch for a full lane; hist_fold_hot adds the
-// lane bins into bin h
-__device__ inline void hist_add32(uint32_t *hist, const uint32_t (&x)[8], uint32_t vl, uint32_t h) {
-    const uint32_t hb = 256u + (threadIdx.x & 31);
-    if (vl >= 32) {
-#pragma unroll
-        for (int q = 0; q < 8; q++)
-#pragma unroll
-            for (int i = 0; i < 4; i++) {
-                const uint32_t v = __byte_perm(x[q], 0u, 0x4440u + i);
-                atomicAdd(&hist[v == h ? hb : v], 1u);
-            }
-    } else {
-#pragma unroll
-        for (int q = 0; q < 8; q++)
-#pragma unroll
-            for (int i = 0; i < 4; i++) {
-                const uint32_t v = __byte_perm(x[q], 0u, 0x4440u + i);
-                if ((uint32_t)(4 * q + i) < vl) atomicAdd(&hist[v == h ? hb : v], 1u);
-            }
-    }
-}
-// the lane bins of hist_add32 into bin h (one warp, after the CTA's counting)
-__device__ inline void hist_fold_hot(uint32_t *hist, uint32_t h) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t c = __reduce_add_sync(0xffffffffu, hist[256 + lane]);
-    if (lane == 0) hist[h] += c;
 }
 
 // Node symbol counts of a histogram h by prefix sums in canonical order: the
@@ -587,14 +554,25 @@ __device__ inline void enc_part(EncSmem &S, const uint8_t *src, uint32_t C, cons
     }
 }
 
-// Counts input bytes [lo, hi) of the block at src into hist (288 zeroed bins;
-// the whole CTA, no barrier).
-__device__ inline void enc_count(const uint8_t *src, uint32_t lo, uint32_t hi, const uint8_t *src_end, uint32_t *hist,
-                                 uint32_t hot) {
-    for (uint32_t kb = lo + 32u * threadIdx.x; kb < hi; kb += 32u * kEncThreads) {
-        uint32_t x[8];
-        ldg32(src + kb, src_end, x);
-        hist_add32(hist, x, min(32u, hi - kb), hot);
+// Counts input bytes [lo, hi) of the block at src into hist (256 zeroed bins;
+// the whole CTA, no barrier): one shared add per byte, by aligned vectors (the
+// order does not matter; equal bytes of a warp's add do not serialise).
+__device__ inline void enc_count(const uint8_t *src, uint32_t lo, uint32_t hi, uint32_t *hist) {
+    const uint32_t t = threadIdx.x, n = hi - lo;
+    const uint8_t *p = src + lo;
+    const uint32_t head = min(n, (uint32_t)(-reinterpret_cast<intptr_t>(p) & 15)), vecs = (n - head) / 16;
+    if (t < head) atomicAdd(&hist[p[t]], 1u);
+    const uint32_t rest = head + 16 * vecs;
+    if (t < n - rest) atomicAdd(&hist[p[rest + t]], 1u);
+    const uint4 *v = reinterpret_cast<const uint4 *>(p + head);
+#pragma unroll 2
+    for (uint32_t i = t; i < vecs; i += kEncThreads) {
+        const uint4 q = __ldg(v + i);
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) atomicAdd(&hist[__byte_perm(w[k], 0u, 0x4440u + c)], 1u);
     }
 }
 
@@ -720,7 +698,7 @@ __device__ inline void encode_item(int b, uint32_t cA, uint32_t share, uint32_t 
             S.end[t] = 8u * L.body_off[t] + L.nv[t] * max(1u, fd);
         }
         if (t < 17) S.first[t] = L.depth_first[t];
-        if (t == 0) { S.maxd = L.max_depth; S.hot = 0xFFFFu; S.bad = 0; }
+        if (t == 0) { S.maxd = L.max_depth; S.bad = 0; }
         {   // byte t: zeros to the front, both sides in order
             uint32_t e = 0, z = 0, o = 8u - __popc((uint32_t)t);
             for (uint32_t j = 0; j < 8; j++) {
@@ -735,8 +713,6 @@ __device__ inline void encode_item(int b, uint32_t cA, uint32_t share, uint32_t 
     const bool big = L.big != 0;
     {
         const uint32_t l = L.len[t];
-        const uint32_t key = __reduce_min_sync(0xffffffffu, l ? (l << 8) | (uint32_t)t : 0xFFFFu);
-        if (lane == 0) atomicMin(&S.hot, key);
         const uint32_t pm = __ballot_sync(0xffffffffu, l != 0);
         if (lane == 0) S.pmask[warp] = pm;
         // a node's bit is one from its right child's first code index on
@@ -746,21 +722,18 @@ __device__ inline void encode_item(int b, uint32_t cA, uint32_t share, uint32_t 
         }
     }
     __syncthreads();   // (the staged layout is dead from here on)
-    const uint32_t hot = S.hot & 0xFFu;
     const uint8_t *src = in + i0;
     const uint8_t *src_end = in + i1;
     uint32_t *rec32 = reinterpret_cast<uint32_t *>(rec);
     // counting scratch in the second level buffer (free between parts)
     uint32_t *hist = reinterpret_cast<uint32_t *>(S.buf[1]);
-    uint32_t *hc = hist + 288, *ps = hist + 544;   // (after the 32 lane bins of the counting)
+    uint32_t *hc = hist + 256, *ps = hist + 512;
     uint32_t acc = 0;              // count of symbol t in the plan chunk's symbols counted so far
     // an item inside a block starts every node's cursor after the symbols before it
     if (!whole && (cA > 0 || share > 0)) {
-        for (int s = t; s < 288; s += kEncThreads) hist[s] = 0;
+        hist[t] = 0;
         __syncthreads();
-        enc_count(src, ch0, P0, src_end, hist, hot);
-        __syncthreads();
-        if (warp == 0) hist_fold_hot(hist, hot);
+        enc_count(src, ch0, P0, hist);
         __syncthreads();
         uint32_t h = hist[t];
         acc = h;
@@ -778,7 +751,7 @@ __device__ inline void encode_item(int b, uint32_t cA, uint32_t share, uint32_t 
     while (P < P1) {
         const uint32_t C = min(len, P1 - P);
         // the part's histogram: the planning pass's chunk counts, or counted here
-        for (int s = t; s < 288; s += kEncThreads) hist[s] = 0;
+        hist[t] = 0;
         __syncthreads();
         const bool given = whole && chunk_hist && C == P1 - P0;
         if (given) {
@@ -786,9 +759,7 @@ __device__ inline void encode_item(int b, uint32_t cA, uint32_t share, uint32_t 
             for (uint32_t c = 0; c < nw; c++) h += __ldg(chunk_hist + ((size_t)b * kEncChunks + c) * 256 + t);
             hist[t] = h;
         } else {
-            enc_count(src, P, P + C, src_end, hist, hot);
-            __syncthreads();
-            if (warp == 0) hist_fold_hot(hist, hot);
+            enc_count(src, P, P + C, hist);
         }
         __syncthreads();
         const uint32_t hcount = hist[t];
