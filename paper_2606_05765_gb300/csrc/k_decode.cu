@@ -914,7 +914,9 @@ cudaError_t read_decode_ws_need(const uint8_t *ws, int nblk, size_t *need, cudaS
 // What bounds it: the latency of a round's chain (state, class, table entry,
 // word), about 380 cycles, 512 rounds a unit whatever its lanes.  2048 blocks
 // of 128 KiB, P(0) = 0.95: 147 us before (one warp per segment, 73
-// instructions a round), 102 us now (48, no branches in a round).
+// instructions a round), 102 us now (48, no branches in a round).  18 blocks of
+// 67842 symbols, a root bitmap of 8.5 KB each: 138 us before, 101 now (153 with
+// the words of a unit that does not fit the shared memory read from the record).
 // ---------------------------------------------------------------------------
 constexpr int kAnsWarps = kDecWarps;
 struct AnsGroup {               // a segment of a unit
@@ -928,7 +930,7 @@ struct AnsGroup {               // a segment of a unit
 struct __align__(16) AnsWarpSm {
     union {
         // per group and class: frequency, start, ceil(2^31 / frequency), class
-        // base; then the groups' words, as far as they fit
+        // base; then windows of the groups' words
         uint4 tab[36][9];
         struct {
             uint4 tab0[9];
@@ -1181,71 +1183,63 @@ __device__ __noinline__ int ans_item(uint32_t g, const uint8_t *__restrict__ com
         AnsStarts st;
 #pragma unroll
         for (int i = 0; i < 4; i++) st.p[i] = tab[2 * i + 1].y | (tab[2 * i + 2].y << 16);
-        // the groups' words into shared memory, group after group, when they
-        // fit beside the tables (they nearly always do: 512 bytes of bitmap a
-        // lane); else the rounds read them from the record
-        uint32_t *area = reinterpret_cast<uint32_t *>(M.tab[ng]);
-        const uint32_t room4 = (uint32_t)(sizeof(M.tab) - sizeof(M.tab[0]) * ng) / 4;
-        uint32_t used = 0;
-        const uint8_t *mine = words;
-        bool staged = false;
-        for (uint32_t i = 0; i < ng; i++) {
-            const int own = (int)M.grp[i].lane0;
-            const uint32_t n2 = __shfl_sync(0xffffffffu, nw, own);
-            const uintptr_t p = (uintptr_t)__shfl_sync(0xffffffffu, (unsigned long long)reinterpret_cast<uintptr_t>(words), own);
-            const uint32_t n4 = (n2 + 1) / 2, sh = 8u * (uint32_t)(p & 3);
-            if (used + n4 > room4) continue;
-            const uint32_t *q = reinterpret_cast<const uint32_t *>(p & ~(uintptr_t)3);
-            const uint32_t *qe = reinterpret_cast<const uint32_t *>(rec + ld_le32(rec));   // (a multiple of 16 bytes)
-            for (uint32_t j = lane; j < n4; j += 32)
-                area[used + j] = __funnelshift_r(q + j < qe ? __ldg(q + j) : 0u, q + j + 1 < qe ? __ldg(q + j + 1) : 0u, sh);
-            if (gi == i) { mine = reinterpret_cast<const uint8_t *>(area + used); staged = true; }
-            used += n4;
-        }
+        // the groups' words go through shared memory: each lane has q4 words of
+        // memory of the space beside the tables (4 at least, 8 stream words),
+        // a group its lanes' together; they are refilled between batches of
+        // four rounds, all groups at once, so that a round has no check and no
+        // branch: every lane takes the step and keeps it while its segment lasts
+        constexpr uint32_t kBatch = 4;
+        static_assert((sizeof(M.tab) - 32 * sizeof(M.tab[0])) / 4 / 32 * 2 >= kBatch, "a batch's words fit");
+        const uint32_t q4 = (uint32_t)(sizeof(M.tab) - sizeof(M.tab[0]) * ng) / 4 / 32;
+        uint32_t *area = reinterpret_cast<uint32_t *>(M.tab[ng]) + q4 * (on ? M.grp[gi].lane0 : 0u);
         const uint16_t *win = reinterpret_cast<const uint16_t *>(area);
-        const uint32_t wofs = staged ? (uint32_t)(mine - reinterpret_cast<const uint8_t *>(area)) / 2 : 0u;
-        __syncwarp();
+        const uint32_t *rend = reinterpret_cast<const uint32_t *>(rec + ld_le32(rec));   // (a multiple of 16 bytes)
         const uint32_t rounds = __reduce_max_sync(0xffffffffu, (sb + nl - 1) / nl);
         const uint32_t mine_r = li < sb ? (sb - li + nl - 1) / nl : 0u;   // this lane's rounds
-        if (__all_sync(0xffffffffu, !on || staged)) {
-            // no branch in a round: every lane takes the step and keeps it while its segment lasts
-            for (uint32_t r0 = 0; r0 < rounds; r0 += 4) {
+        uint32_t wbase = 0, wlim = 0;   // the group's words wbase .. wlim - 1 are staged
+        uint8_t *o = dst + li;
+        for (uint32_t r0 = 0; r0 < rounds; r0 += kBatch, o += kBatch * nl) {
+            if (__any_sync(0xffffffffu, rd + kBatch * nl > wlim && wlim < nw)) {
+                __syncwarp();
+                // (here rd <= wlim <= nw: a batch takes kBatch nl words at most)
+                const uint8_t *p = words + 2ull * rd;
+                const uint32_t sh = 8u * (uint32_t)(reinterpret_cast<uintptr_t>(p) & 3), n = min(2 * q4 * nl, nw - min(rd, nw));
+                const uint32_t *q = reinterpret_cast<const uint32_t *>(p - sh / 8);
+                if (rd <= nw) {
+#pragma unroll 8
+                    for (uint32_t i = li; i < (n + 1) / 2; i += nl)
+                        area[i] = __funnelshift_r(q + i < rend ? __ldg(q + i) : 0u, q + i + 1 < rend ? __ldg(q + i + 1) : 0u, sh);
+                    wbase = rd;
+                    wlim = rd + n;
+                }
+                __syncwarp();
+            }
+            uint32_t at[kBatch];
+#pragma unroll
+            for (uint32_t j = 0; j < kBatch; j++) {
+                const bool active = r0 + j < mine_r;
+                uint32_t xn = x;
+                at[j] = ans_step(tab, st, xn);
+                const bool need = active && xn < kAnsL;
+                const uint32_t m = __ballot_sync(0xffffffffu, need) & gm;
+                // (past the last word the count below is off and the stream refused)
+                const uint32_t y = (xn << 16) | win[min(rd + __popc(m & lt), wlim) - wbase];
+                x = active ? (need ? y : xn) : x;
+                rd += __popc(m);
+            }
+            uint32_t by[kBatch];
+#pragma unroll
+            for (uint32_t j = 0; j < kBatch; j++) by[j] = I.member[at[j]] ^ xr;
+            // a single lane's bytes follow one another: whole words (past the end: the zeros)
+            if (nl == 1) {
                 uint32_t acc = 0;
 #pragma unroll
-                for (uint32_t j = 0; j < 4; j++) {
-                    const uint32_t r = r0 + j;
-                    const bool active = r < mine_r;
-                    uint32_t xn = x;
-                    const uint32_t by = I.member[ans_step(tab, st, xn)] ^ xr;
-                    const bool need = active && xn < kAnsL;
-                    const uint32_t m = __ballot_sync(0xffffffffu, need) & gm;
-                    // (past the last word the count below is off and the stream refused)
-                    const uint32_t y = (xn << 16) | win[wofs + min(rd + __popc(m & lt), nw)];
-                    x = active ? (need ? y : xn) : x;
-                    rd += __popc(m);
-                    acc |= active ? by << (8 * j) : 0u;
-                    if (nl > 1 && active) dst[r * nl + li] = (uint8_t)by;
-                }
-                // a single lane's bytes follow one another: whole words (past the end: the zeros)
-                if (nl == 1 && r0 < mine_r) *reinterpret_cast<uint32_t *>(dst + r0) = acc;
-            }
-        } else {
-            for (uint32_t r = 0; r < rounds; r++) {
-                const bool active = r < mine_r;
-                uint32_t by = 0;
-                bool need = false;
-                if (active) {
-                    by = I.member[ans_step(tab, st, x)] ^ xr;
-                    need = x < kAnsL;
-                }
-                const uint32_t m = __ballot_sync(0xffffffffu, need) & gm, pos = rd + __popc(m & lt);
-                if (need) {
-                    if (pos >= nw) ok = false;
-                    else if (staged) x = (x << 16) | win[wofs + pos];
-                    else x = (x << 16) | (uint32_t)__ldg(words + 2 * pos) | ((uint32_t)__ldg(words + 2 * pos + 1) << 8);
-                }
-                rd += __popc(m);
-                if (active) dst[r * nl + li] = (uint8_t)by;
+                for (uint32_t j = 0; j < kBatch; j++) acc |= r0 + j < mine_r ? by[j] << (8 * j) : 0u;
+                if (r0 < mine_r) *reinterpret_cast<uint32_t *>(dst + r0) = acc;
+            } else {
+#pragma unroll
+                for (uint32_t j = 0; j < kBatch; j++)
+                    if (r0 + j < mine_r) o[j * nl] = (uint8_t)by[j];
             }
         }
     }

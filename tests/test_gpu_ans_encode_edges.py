@@ -1,5 +1,5 @@
-"""GPU: ANS-coded records byte for byte against the oracle at the sizes where
-the units of the ANS encode meet: bitmaps of one byte to several 16 KiB
+"""GPU: ANS-coded records byte for byte against the oracle, and decoded again,
+at the sizes where the units of the ANS coder meet: bitmaps of one byte to several 16 KiB
 segments, last segments too short to hold their own states (or that grow when
 coded), nodes kept raw between coded ones, and a scratch buffer with no room
 for the last block's mirror (one warp codes that block)."""
@@ -23,6 +23,8 @@ def blocks_of(kind, rng):
     if kind == "segments":
         return bitmap_blocks(rng, [16383, 16384] + [16384 + k for k in (1, 2, 3, 5, 9, 13, 16, 17, 31, 40, 511, 513, 8191)]
                              + [32767, 32768, 32769, 32768 + 15])
+    if kind == "dense":     # bitmaps that hardly compress: more words than a unit's windows hold at once
+        return [draw(rng, 8 * s, p, 2) for s in (300, 600, 3000, 8480, 8704, 12000, 16383) for p in (0.72, 0.8)]
     if kind == "growing":   # the last segment, or a whole one, does not compress
         out = []
         for n, m in ((16384, 20), (16384, 700), (16384, 4000), (32768, 11000), (16384, 16384), (32768, 16384 + 300)):
@@ -34,7 +36,7 @@ def blocks_of(kind, rng):
             for _ in range(40)] + [draw(rng, 300000, 0.9, 30)]
 
 
-@pytest.mark.parametrize("kind", ["tiny", "segments", "growing", "nodes"])
+@pytest.mark.parametrize("kind", ["tiny", "segments", "dense", "growing", "nodes"])
 def test_ans_encode_edges(P, kind):   # noqa: F811
     import oracle
     oracle.build()
@@ -56,3 +58,7 @@ def test_ans_encode_edges(P, kind):   # noqa: F811
         for b in range(n):
             assert rb[b] == sizes[b], (kind, room < total, b)
             assert np.array_equal(comp[eo[b]:eo[b] + rb[b]], ref[int(rec_off[b]):int(rec_off[b]) + int(sizes[b])]), (kind, b)
+    for batched in (False, True):
+        out, st = P.decode(e.comp, e.off, off64(off), batched=batched)
+        assert not st.cpu().numpy().any()
+        assert np.array_equal(out.cpu().numpy()[: data.size], data), (kind, batched)
