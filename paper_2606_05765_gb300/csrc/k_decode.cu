@@ -1407,24 +1407,25 @@ __device__ inline BitLd tile_ld(const TileSrc &s, uint32_t pos, uint32_t k) {
 __device__ inline uint32_t tile_word(const BitLd &b) { return __funnelshift_r(b.lo, b.hi, b.sh); }
 __device__ inline uint32_t tile_bits(const TileSrc &s, uint32_t pos, uint32_t k) { return tile_word(tile_ld(s, pos, k)); }
 
-// popcount of bits [e, e + len) (len <= 256) of the bitmap at bit address
-// pos: the covering words are loaded together, then counted
-__device__ inline uint32_t tile_popc(const TileSrc &s, uint32_t pos, uint32_t e, uint32_t len) {
+// popcount of bits [e, e + len) (len <= 32 (kW - 1)) of the bitmap at bit
+// address pos: the covering words are loaded together, then counted
+template <int kW>
+__device__ inline uint32_t tile_popc_w(const TileSrc &s, uint32_t pos, uint32_t e, uint32_t len) {
     const bool sc = (pos >> 31) != 0;
     const uint64_t a = (uint64_t)(pos & 0x7FFFFFFFu) + e;
     const uint64_t w0 = a >> 5;
     const uint32_t sh = (uint32_t)a & 31u;
     const uint32_t *w = reinterpret_cast<const uint32_t *>(sc ? s.scr : s.rec);
     const uint64_t lim = sc ? s.scr_bytes : (uint64_t)s.rec_bytes;
-    const uint32_t nw = (sh + len + 31) >> 5;   // words holding the range (<= 9)
-    uint32_t x[9];
+    const uint32_t nw = (sh + len + 31) >> 5;   // words holding the range (<= kW)
+    uint32_t x[kW];
 #pragma unroll
-    for (int i = 0; i < 9; i++) x[i] = ((uint32_t)i < nw && 4 * (w0 + i) + 4 <= lim) ? __ldcg(w + w0 + i) : 0u;
+    for (int i = 0; i < kW; i++) x[i] = ((uint32_t)i < nw && 4 * (w0 + i) + 4 <= lim) ? __ldcg(w + w0 + i) : 0u;
     // all bits of the loaded words, less those before sh in the first and
     // those from sh + len on in the last
     uint32_t c = 0, xl = 0;
 #pragma unroll
-    for (int i = 0; i < 9; i++) {
+    for (int i = 0; i < kW; i++) {
         c += __popc(x[i]);
         xl = (uint32_t)i + 1 == nw ? x[i] : xl;
     }
@@ -1432,6 +1433,10 @@ __device__ inline uint32_t tile_popc(const TileSrc &s, uint32_t pos, uint32_t e,
     const uint32_t eb = (sh + len) & 31u;
     if (eb) c -= __popc(xl >> eb);
     return c;
+}
+// (len <= 256; directories are built and used with fewer bits than that, as a rule 128)
+__device__ inline uint32_t tile_popc(const TileSrc &s, uint32_t pos, uint32_t e, uint32_t len) {
+    return tile_popc_w<9>(s, pos, e, len);
 }
 
 // 8 bytes of a level buffer from byte a (reads up to 11 bytes past a)
@@ -2017,8 +2022,8 @@ __device__ __noinline__ void tile_close(int how, const uint8_t *__restrict__ com
 //             shares between the node's start and the entry
 // What bounds them: the latency of dependent reads (a share's windows one
 // after another, a boundary's levels one after another).  One CTA per block
-// took 242 us for a block of 2^20 symbols alone; shares and cursors take 34 +
-// 24 us.
+// took 242 us for a block of 2^20 symbols alone; shares and cursors take 44 +
+// 29 us.
 // ---------------------------------------------------------------------------
 constexpr uint32_t kDirShares = 128;   // shares of a block at most
 constexpr uint32_t kDirShareMin = 10;  // log2 of the fewest entries of a share (but for the block's last)
@@ -2080,6 +2085,7 @@ __device__ inline bool dir_ref(int b, uint32_t k, const uint8_t *__restrict__ co
     const uint32_t *nsrc = reinterpret_cast<const uint32_t *>(nt + kNtabHdr);
     const uint32_t *nv = reinterpret_cast<const uint32_t *>(rec + kNvOff);
     __syncwarp();
+#pragma unroll 4
     for (uint32_t v = lane; v < D.V; v += 32) {
         M.nv[v] = __ldg(nv + v);
         M.src[v] = nsrc[3 * v];
@@ -2092,15 +2098,13 @@ __device__ inline bool dir_ref(int b, uint32_t k, const uint8_t *__restrict__ co
     return true;
 }
 
-// Share k of block b's directory (one warp).
-__device__ __noinline__ void dir_share(int b, uint32_t k, const uint8_t *__restrict__ comp,
-                                       const uint64_t *__restrict__ comp_off, int nblk, uint8_t *__restrict__ ws,
-                                       uint64_t ws_bytes, int32_t *__restrict__ status) {
+// Share k of block b's directory (one warp): superblocks of dir_bits, whose
+// bits lie in kW words at most (five for the 128 bits of the default: 509
+// text-like blocks 52 us with nine, 47 with five).
+template <int kW>
+__device__ inline void dir_share_count(const DirRef &D, const DirWarpSm &M, uint32_t k, uint32_t dir_bits) {
     const int lane = threadIdx.x & 31;
-    DirWarpSm &M = (&smem_item<DirWarpSm>())[threadIdx.x >> 5];
-    DirRef D;
-    if (!dir_ref(b, k, comp, comp_off, nblk, ws, ws_bytes, status, M, D) || k >= D.shares) return;
-    const uint32_t dir_bits = dec_dir_bits(ws), V = D.V;
+    const uint32_t V = D.V;
     const uint32_t g0 = k << D.slog, g1 = min(D.ent, g0 + (1u << D.slog));
     const uint32_t le = 0xFFFFFFFFu >> (31 - lane);
     uint32_t vcur = (uint32_t)find_node_d(M.u, 0, (int)V, g0), carry = 0;
@@ -2128,7 +2132,7 @@ __device__ __noinline__ void dir_share(int b, uint32_t k, const uint8_t *__restr
             if (g < g1) {
                 const uint32_t v = vv[r], e0 = (g - M.u[v]) * dir_bits;
                 // (a flat node's body is indices: its superblocks are not read)
-                if (e0 < M.nv[v] && !ch_flat_d(M.ch[v])) pc[r] = tile_popc(D.src, M.src[v], e0, min(dir_bits, M.nv[v] - e0));
+                if (e0 < M.nv[v] && !ch_flat_d(M.ch[v])) pc[r] = tile_popc_w<kW>(D.src, M.src[v], e0, min(dir_bits, M.nv[v] - e0));
             }
         }
 #pragma unroll
@@ -2144,6 +2148,16 @@ __device__ __noinline__ void dir_share(int b, uint32_t k, const uint8_t *__restr
         }
     }
     if (lane == 0) D.cur[(size_t)k * V] = carry;
+}
+__device__ __noinline__ void dir_share(int b, uint32_t k, const uint8_t *__restrict__ comp,
+                                       const uint64_t *__restrict__ comp_off, int nblk, uint8_t *__restrict__ ws,
+                                       uint64_t ws_bytes, int32_t *__restrict__ status) {
+    DirWarpSm &M = (&smem_item<DirWarpSm>())[threadIdx.x >> 5];
+    DirRef D;
+    if (!dir_ref(b, k, comp, comp_off, nblk, ws, ws_bytes, status, M, D) || k >= D.shares) return;
+    const uint32_t dir_bits = dec_dir_bits(ws);
+    if (dir_bits <= 128) dir_share_count<5>(D, M, k, dir_bits);
+    else dir_share_count<9>(D, M, k, dir_bits);
 }
 
 // Cursors of block b at tile boundary k (1 <= k < ntile), after all the
