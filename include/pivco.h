@@ -153,25 +153,26 @@ pivco_status pivco_encode_blocks(const uint8_t *in, const uint64_t *blk_off, int
                                  void *layout, uint8_t *out, const uint64_t *out_off,
                                  uint64_t *rec_bytes, int32_t *status, void *stream);
 
-/* The encoder's warp chunks counted in the histogram pass.  Block b of n
+/* The encoder's chunks counted in the histogram pass.  Block b of n
  * symbols is cut into nw = min(8, max(1, n / 4096)) contiguous chunks, chunk
- * w starting at floor(n w / nw) rounded down to a multiple of 32 (the split
- * pivco_encode_blocks uses for its warps).  pivco_histogram_chunks writes the
+ * w starting at floor(n w / nw) rounded down to a multiple of 32.
+ * pivco_histogram_chunks writes the
  * block histograms to hist[nblk][256] exactly as pivco_histogram does, and
  * each chunk's histogram to chunk_hist[nblk][8][256] (device; the chunks a
  * block does not have are zeros).  pivco_encode_blocks_chunked is
  * pivco_encode_blocks reading those chunk histograms instead of counting the
  * chunks again; the records are byte-identical.  The encoder codes a block
- * in runs of consecutive chunks whose levels fit its buffers, taking each
- * run's node counts from the summed chunk histograms (a chunk too large for
- * the buffers is coded in parts counted from `in`, and the parts' counts
- * must add up to its histogram).  Chunk histograms that do not describe
+ * whose levels fit its buffers in one part, taking the node counts from the
+ * summed chunk histograms (a block too large for the buffers is coded in
+ * parts counted from `in`, and the parts' counts must add up to the chunks'
+ * histograms).  Chunk histograms that do not describe
  * `in` (another input, or stale) never give a wrong record with an OK
  * status: a block is either refused (status[b] = PIVCO_ERR_INVALID_ARG) or,
  * when the sums it used are right after all, encoded exactly; nothing is
  * written outside each block's record.  A block whose levels do not fit
- * the encoder's buffers is coded chunk by chunk by several CTAs (a work
- * list of (block, chunk) items); each chunk starts at the node cursors its
+ * the encoder's buffers, or one of 16384 symbols and more in a batch of few
+ * blocks, is coded chunk by chunk by several CTAs (a work list of (block,
+ * chunk) items, or shares of chunks); each chunk starts at the node cursors its
  * preceding chunks' histograms give.  Both encode calls keep that work list
  * in scratch words at the end of the layout records, so one layout serves
  * one encode call at a time. */
@@ -298,9 +299,11 @@ pivco_status pivco_server_destroy(pivco_server *srv);
  *                       places the ANS work in `ws` (single-pass scan with
  *                       decoupled look-back over the blocks); sets status[b];
  *   pivco_decode_ans    rANS-decodes every ANS-coded node bitmap into the
- *                       workspace (Sec. 5.2), one warp per 16 KiB segment;
+ *                       workspace (Sec. 5.2), one warp per 16 KiB segment,
+ *                       shorter segments sharing warps;
  *   pivco_decode_merge  rebuilds the symbols bottom-up (Sec. 3) through
- *                       per-chunk rank directories, one CTA per block. */
+ *                       rank directories at tile boundaries, one CTA per
+ *                       tile. */
 pivco_status pivco_decode_plan(const uint8_t *comp, const uint64_t *comp_off, int32_t nblk, void *ws,
                                size_t ws_bytes, int32_t *status, void *stream);
 pivco_status pivco_decode_ans(const uint8_t *comp, const uint64_t *comp_off, int32_t nblk, void *ws,
@@ -387,10 +390,11 @@ uint64_t pivco_get_wait_limit(void);
 /* ---- Batching (not in the paper: the GPU scheduling of many blocks) ----
  * pivco_decode_batched decodes the same records as pivco_decode_blocks (same
  * arguments, same workspace size, identical output) with one persistent
- * launch whose work queue is keyed by (block, stage): record plans, first
- * tiles (the only tile of a block that needs no ANS segment and no
- * directory, as soon as its own plan is complete), ANS segments, rank
- * directories, the other tiles.  Each item waits (bounded, by default 1 s)
+ * launch whose work queue is keyed by (block, stage): the blocks (a block
+ * of one tile that needs no ANS segment and no directory is decoded here, as
+ * soon as its own plan is complete; large batches plan several blocks to an
+ * item first), ANS segments, rank directories, the other tiles.  Each item
+ * waits (bounded, by default 1 s)
  * only on items earlier in the queue; an expired wait marks the block
  * PIVCO_ERR_TIMEOUT. */
 pivco_status pivco_decode_batched(const uint8_t *comp, const uint64_t *comp_off, int32_t nblk,

@@ -699,7 +699,7 @@ __device__ inline void plan_rest(int b, int nblk, int max_len, const SelectParam
 
 static_assert(kHistThreads == kPmThreads && kPmThreads == kLayThreads, "one CTA shape for the three steps");
 
-__global__ void __launch_bounds__(kHistThreads) block_plan_kernel(
+__global__ void __launch_bounds__(kHistThreads, 8) block_plan_kernel(
     const uint8_t *__restrict__ in, const uint64_t *__restrict__ blk_off, int max_len,
     const __grid_constant__ SelectParams sp, uint32_t *__restrict__ hist, uint32_t *__restrict__ chunk_hist,
     uint8_t *__restrict__ lens_out, BlockLayout *__restrict__ layout, uint64_t *__restrict__ rec_bound,

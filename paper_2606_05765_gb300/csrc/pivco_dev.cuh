@@ -296,8 +296,10 @@ __device__ inline void flat_tree_build(const int32_t *cnt, const int32_t *start,
     // rank of an item among the items of its length, by first symbol
     for (int i = lane; i < n; i += 32) {
         const uint32_t fs = sorted[F.iso[i]];
+        const uint32_t l = F.il[i];
         int r = 0;
-        for (int j = 0; j < n; j++) r += F.il[j] == F.il[i] && sorted[F.iso[j]] < fs;
+#pragma unroll 4
+        for (int j = 0; j < n; j++) r += (uint32_t)(F.il[j] == l) & (uint32_t)(sorted[F.iso[j]] < fs);
         F.irank[i] = (uint8_t)r;
         if (r < 9) F.it_of[F.il[i]][r] = (uint8_t)i;
         else ok = false;
@@ -342,9 +344,10 @@ __device__ inline void flat_tree_build(const int32_t *cnt, const int32_t *start,
     // before each one
     if (ok) {
         for (int i = lane; i < n; i += 32) {
+            const uint32_t key = F.il[i] * 16u + F.irank[i];   // (ranks are below 9)
             uint32_t off = 0;
-            for (int j = 0; j < n; j++)
-                if (F.il[j] < F.il[i] || (F.il[j] == F.il[i] && F.irank[j] < F.irank[i])) off += 1u << F.iD[j];
+#pragma unroll 4
+            for (int j = 0; j < n; j++) off += F.il[j] * 16u + F.irank[j] < key ? 1u << F.iD[j] : 0u;
             F.ioff[i] = (uint16_t)off;
         }
     }
@@ -430,16 +433,17 @@ void count_launches(int n);
 inline int div_up(long long a, long long b) { return (int)((a + b - 1) / b); }
 
 // Launchers implemented in the kernel translation units.
-// Warp chunks of an encoded block: a block of n symbols is cut into
+// Chunks of an encoded block: a block of n symbols is cut into
 // nw = min(8, max(1, n / 4096)) contiguous chunks, chunk w starting at
-// floor(n w / nw) rounded down to a multiple of 32.  The encoder gives chunk w
-// to its warp w; the chunked histogram counts each chunk on its own.
+// floor(n w / nw) rounded down to a multiple of 32.  The chunked histogram
+// counts each chunk on its own; the chunks of a big block are coded by
+// several CTAs.
 constexpr uint32_t kEncChunks = 8;
 constexpr int kEBuf = 22016;         // symbols per encoder level buffer (4 CTAs per SM)
 constexpr uint32_t kEncShares = 8;   // shares of a chunk at most
 // Batches of at most this many blocks split their blocks of at least this
-// size over several CTAs (26 blocks of 39-79 KB: 162 us by one CTA each,
-// 124 us by chunks)
+// size over several CTAs (26 blocks of 39-79 KB, plan to ANS: 162 us by one CTA
+// each, 124 us by chunks)
 constexpr uint32_t kEncFewBlocks = 152, kEncFewSize = 16384;
 constexpr uint32_t kEncMinChunk = 4096;
 __host__ __device__ inline uint32_t enc_nchunks(uint64_t n) {
@@ -477,17 +481,18 @@ cudaError_t launch_ans_decode(const uint8_t *bodies, const uint64_t *body_off, c
                               uint8_t *bm, const uint64_t *bm_off, int32_t *status, cudaStream_t st);
 // ---------------------------------------------------------------------------
 // Decode workspace (written by the decode plan, read by the later passes):
-//   header (64 B): u64 scratch bytes @0, u32 ANS segments @8, u32 ticket @12,
+//   header (64 B): u64 scratch bytes @0, u32 ANS units @8,
 //                  u64 directory+cursor bytes @16, u32 tiles @24,
 //                  u32 directory granularity (bits) @28, u32 longest tile @32,
 //                  u32 batch queue ticket @36, u32 batch plans done @40,
-//                  u32 items done (serving) @44, u32 tile ticket @48,
+//                  u32 items done (serving) @44, u32 tile ticket @48 (batched: the
+//                  blocks left for the tile stage),
 //                  u32 abandoned @52 (a CTA gave up on the queue),
 //                  u64 wait bound in ns @56
 //   per block: u64 look-back states A[nblk], B[nblk]; u64 scratch offset[nblk];
-//              u64 directory offset[nblk]; u32 first segment[nblk];
+//              u64 directory offset[nblk]; u32 first ANS unit[nblk];
 //              u32 first tile[nblk]; u32 tile length[nblk]; u32 tiles[nblk];
-//              u32 ANS segments done[nblk]; u32 directory done[nblk]
+//              u32 ANS units done[nblk]; u32 directory items done[nblk]; u32 plan done[nblk]
 //   then: rank directories and tile-boundary cursors, ANS-decoded bitmaps.
 // ---------------------------------------------------------------------------
 struct DecWs {
