@@ -680,11 +680,12 @@ struct PlanSmem {
     } u;
 };
 
-// Batches of at most one block per SM run as clusters of one CTA per chunk: a
-// block of at least kPlanWide symbols is counted by all eight, a smaller one
-// by the first.  (One block of 1 MiB: 93 us by one CTA, 35 us by eight; 509
-// text-like blocks 57 and 62 us, 1024 mixed blocks 135 and 125 us: with blocks
-// enough for every SM the extra CTAs' coming and going takes what they save.)
+// Batches small enough to give every CTA of their clusters an SM of its own run
+// as clusters of one CTA per chunk: a block of at least kPlanWide symbols is
+// counted by all eight, a smaller one by the first.  (One block of 1 MiB: 93 us
+// by one CTA, 35 us by eight; 122 blocks of 75 KB both ways 201 us by one each,
+// 205 by clusters; 509 text-like blocks 57 and 62 us, 1024 mixed blocks 135 and
+// 125 us of the plan: there the extra CTAs' coming and going takes what they save.)
 constexpr uint32_t kPlanWide = 32768;
 
 __device__ inline void plan_rest(int b, int nblk, int max_len, const SelectParams &sp, PlanSmem &P,
@@ -746,7 +747,7 @@ cudaError_t launch_block_plan(const uint8_t *in, const uint64_t *blk_off, int nb
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (nblk <= sms)
+    if (nblk * (int)kEncChunks <= sms)
         block_plan_cluster_kernel<<<nblk * (int)kEncChunks, kHistThreads, 0, st>>>(in, blk_off, p.max_len, sp, hist, chunk_hist,
                                                                                     lens, layout, rec_bound, status);
     else

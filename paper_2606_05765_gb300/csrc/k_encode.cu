@@ -27,8 +27,8 @@
 // What bounds it: instruction issue and shared-memory wavefronts.  (With 32
 // symbols of 16 bits to a lane, a window took about 800 instructions and 200
 // wavefronts.)  Before and now: 2048 blocks of 128 KiB, 350 -> 283 us; the
-// chunks of one block of 1 MiB, 330 -> 89 us, and of 509 text-like blocks, 564
-// -> 436 us; 4096 blocks of 64 KiB, whose root has a leaf child, 439 -> 435 us.
+// chunks of one block of 1 MiB, 330 -> 52 us, and of 509 text-like blocks, 564
+// -> 361 us; 4096 blocks of 64 KiB, whose root has a leaf child, 439 -> 403 us.
 
 #include "levels.cuh"
 
@@ -890,8 +890,11 @@ __device__ inline void enc_list_place(uint32_t i, uint32_t len, const uint64_t *
         }
         place += __syncthreads_count(before);
     }
-    if (threadIdx.x == 0)
-        const_cast<BlockLayout *>(layout_of(layout, place))->list_sorted = layout_of(layout, (int)i)->list_entry;
+    if (threadIdx.x == 0) {
+        __stcg(&const_cast<BlockLayout *>(layout_of(layout, place))->list_sorted, layout_of(layout, (int)i)->list_entry);
+        __threadfence();
+    }
+    __syncthreads();
 }
 
 // One CTA per block (a big block of a chunked encode is left to the chunk
@@ -909,6 +912,8 @@ __global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm) encode_kernel(cons
     if (chunk_hist) {
         const uint32_t len = layout->list_len;
         if (blockIdx.x < len && len <= kEncSortMax) enc_list_place(blockIdx.x, len, blk_off, layout);
+        // (the chunk kernel may start from here on)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         if (layout_of(layout, (int)blockIdx.x)->big) return;
     }
     encode_item<true>((int)blockIdx.x, 0, 0, 1, in, blk_off, layout, chunk_hist, out, out_off, rec_bytes, status, S);
@@ -929,22 +934,32 @@ __global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm) encode_chunks_kern
     extern __shared__ __align__(128) uint8_t smem_raw[];
     EncSmem &S = *reinterpret_cast<EncSmem *>(smem_raw);
     __shared__ uint32_t s_tk;
-    const uint32_t len = layout->list_len, chunks = len * kEncChunks;
-    if (chunks == 0) return;
-    const uint32_t shares = min(kEncShares, max(1u, gridDim.x / chunks)), items = chunks * shares;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_tk = atomicAdd(&layout->list_ticket, 1u);
-        __syncthreads();
-        const uint32_t tk = s_tk;
-        if (tk >= items) return;
+    // (the list and its order are complete: all of encode_kernel's CTAs are past writing them)
+    const uint32_t len = __ldcg(&layout->list_len), chunks = len * kEncChunks;
+    const uint32_t shares = min(kEncShares, max(1u, gridDim.x / max(1u, chunks))), items = chunks * shares;
+    // an item each: by the CTA's number, which the launch deals out over the SMs (tickets taken in the order
+    // of arrival put four of the 64 shares of one block on some SMs and none on others: 85 us, 52 spread).
+    // More items: by ticket, the largest first to whoever comes first.
+    const bool each = items <= gridDim.x;
+    uint32_t tk = blockIdx.x;
+    while (chunks) {
+        if (!each) {
+            __syncthreads();
+            if (threadIdx.x == 0) s_tk = atomicAdd(&layout->list_ticket, 1u);
+            __syncthreads();
+            tk = s_tk;
+        }
+        if (tk >= items) break;
         const BlockLayout *E = layout_of(layout, (int)(tk / (kEncChunks * shares)));
-        const int bb = (int)(len <= kEncSortMax ? E->list_sorted : E->list_entry);
+        const int bb = (int)__ldcg(len <= kEncSortMax ? &E->list_sorted : &E->list_entry);
         const uint32_t c = tk / shares % kEncChunks;
         if (c < enc_nchunks(blk_off[bb + 1] - blk_off[bb]))
             encode_item<false>(bb, c, tk % shares, shares, in, blk_off, layout, chunk_hist, out, out_off, rec_bytes,
                                status, S);
+        if (each) break;
     }
+    // what follows in the stream follows encode_kernel too (one CTA waits, the others leave their slots)
+    if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 cudaError_t launch_encode(const uint8_t *in, const uint64_t *blk_off, int nblk, BlockLayout *layout,
@@ -973,8 +988,21 @@ cudaError_t launch_encode(const uint8_t *in, const uint64_t *blk_off, int nblk, 
         const int smem_big = (int)sizeof(EncSmem);
         e = cudaFuncSetAttribute(encode_chunks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_big);
         if (e != cudaSuccess) return e;
-        encode_chunks_kernel<<<sms * kEncCtasPerSm, kEncThreads, smem_big, st>>>(in, blk_off, layout, chunk_hist,
-                                                                                      out, out_off, rec_bytes, status);
+        // started while encode_kernel's last blocks run: its CTAs take the slots that fall free (509 text-like
+        // blocks both ways 807 -> 760 us, 1024 mixed blocks 1297 -> 1205); with a block per SM at most there
+        // is nothing to overlap
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(sms * kEncCtasPerSm);
+        cfg.blockDim = dim3(kEncThreads);
+        cfg.dynamicSmemBytes = (size_t)smem_big;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = nblk > sms ? 1 : 0;
+        e = cudaLaunchKernelEx(&cfg, encode_chunks_kernel, in, blk_off, layout, chunk_hist, out, out_off, rec_bytes, status);
+        if (e != cudaSuccess) return e;
         count_launches(1);
     }
     return cudaGetLastError();
