@@ -1333,7 +1333,7 @@ struct __align__(16) CtaTile {
     uint32_t pos[256];                         // bit address of node v's next bit (bit 31: in the ANS scratch)
     uint32_t dem[256];                         // bits of node v in the current chunk
     uint32_t ch[256];                          // children (node table format)
-    uint32_t src0[256];                        // pos at the start (batch_block)
+    uint32_t end[256];                         // bit address of the end of node v's bits in the tile
     uint32_t strip[kStripMax];                 // ones of the root before each strip of windows
     uint32_t wtot[2][kTileWarps];              // ones of a round's ordinary windows, two rounds deep
     uint16_t sp[256];                          // byte offset of node v's sequence in its level buffer
@@ -1382,9 +1382,10 @@ __device__ inline void sel_init(uint32_t *sel) {
 
 // The two words under 32 bits of a node bitmap from bit address pos + k (bit
 // 31 of pos: scratch), loaded ahead of their use.  The bits lie inside the
-// node's body (the plan has checked the bodies against the record, and a
-// tile's cursors against the bodies), so only the second word can run past
-// the end; bit addresses stay below 2^31.
+// node's body (the plan has checked the bodies against the record, the tile
+// its cursors against the bodies, and ct_demand the demands of a shorter
+// chunk against the tile's end cursors before anything of it is read), so
+// only the second word can run past the end; bit addresses stay below 2^31.
 struct BitLd {
     uint32_t lo, hi, sh;
 };
@@ -1495,9 +1496,9 @@ __device__ inline void merge_window(const uint8_t *bin, uint32_t w, uint32_t a, 
 }
 
 // 8 output symbols of a flat node (Sec. 2.2.3, merge_flat_D): the D-bit
-// indices at bit address pos (a raw body in the record), each mapped through
-// the node's symbols tab[0 .. 2^D).  Neighbouring lanes read neighbouring
-// bytes.
+// indices at bit address pos (a raw body in the record; the first index lies
+// inside it, as for tile_ld), each mapped through the node's symbols
+// tab[0 .. 2^D).  Neighbouring lanes read neighbouring bytes.
 __device__ inline uint2 flat8(const TileSrc &s, uint32_t D, uint32_t pos, const uint8_t *tab) {
     const uint32_t e = pos & 0x7FFFFFFFu, wi = e >> 5, lim = s.rec_bytes >> 2;
     const uint32_t *w = reinterpret_cast<const uint32_t *>(s.rec) + wi;
@@ -1556,16 +1557,19 @@ __device__ inline void put_step(uint8_t *dst, int s, uint2 o, uint32_t nb, uint3
 
 // Demands of a chunk of C root symbols from the current cursors, top-down:
 // a node's popcount over its range splits its demand between its children
-// (one warp).
-__device__ inline void ct_demand(CtaTile &S, const TileSrc &src, uint32_t V, uint32_t C) {
+// (one warp).  False when a node's demand runs past its bits in the tile (the
+// bitmaps above it are corrupt): it is found before the node is read, here
+// or by the levels.
+__device__ inline bool ct_demand(CtaTile &S, const TileSrc &src, uint32_t V, uint32_t C) {
     const int lane = threadIdx.x & 31;
     for (uint32_t v = lane; v < V; v += 32) S.dem[v] = 0;
     __syncwarp();
     if (lane == 0) S.dem[0] = C;
     __syncwarp();
     for (uint32_t v = 0; v < V; v++) {   // breadth-first: parents before children
-        if (ch_flat_d(S.ch[v])) continue;   // a flat node has no children to split for
-        const uint32_t dv = S.dem[v];
+        const uint32_t dv = S.dem[v], fD = ch_flat_d(S.ch[v]);
+        if ((uint64_t)dv * max(1u, fD) > S.end[v] - S.pos[v]) return false;   // (the same in all lanes)
+        if (fD) continue;   // a flat node has no children to split for
         uint32_t ones = 0;
         for (uint32_t e = 32 * lane; e < dv; e += 1024) {
             uint32_t w = tile_bits(src, S.pos[v], e);
@@ -1581,6 +1585,7 @@ __device__ inline void ct_demand(CtaTile &S, const TileSrc &src, uint32_t V, uin
         }
         __syncwarp();
     }
+    return true;
 }
 
 // windows per strip of the root (so that there are at most kStripMax strips)
@@ -1804,8 +1809,8 @@ __device__ inline void cta_fill(uint8_t *p, uint32_t n, uint8_t x) {
 }
 
 // Decodes root symbols [P0, P1) into dst + P0 with the whole CTA: the tables
-// (first, maxd, ftab, pos, dem, ch; the demands of the whole tile) are in S
-// and checked.  kTileBad when the bitmaps are corrupt; kTileChunked when the
+// (first, maxd, ftab, pos, end, dem, ch; the demands of the whole tile) are in
+// S and checked.  kTileBad when the bitmaps are corrupt; kTileChunked when the
 // tile went in several chunks, whose end the caller checks.
 enum : int { kTileBad = 0, kTileOk = 1, kTileChunked = 2 };
 __device__ __forceinline__ int ct_decode() {
@@ -1820,8 +1825,8 @@ __device__ __forceinline__ int ct_decode() {
     // the whole tile at once when its levels fit, else chunks found top-down
     while (P < P1) {
         if (chunked) {
-            if (warp == 0) ct_demand(S, src, V, C);
-            __syncthreads();
+            const bool over = warp == 0 && !ct_demand(S, src, V, C);
+            if (__syncthreads_or(over)) return kTileBad;
         }
         if (!lvl_layout(S)) {
             chunked = true;
@@ -1954,6 +1959,7 @@ __device__ __noinline__ bool tile_open(uint32_t gt, const uint8_t *__restrict__ 
             (bpe > 1 && ((s0 >> 31) || (chv & 0xFFu) + (1u << bpe) > 256u)))
             bad = 1;
         S.pos[v] = s0 + cs * bpe;
+        S.end[v] = s0 + ce * bpe;
         S.dem[v] = ce - cs;
         S.ch[v] = chv;
     }
@@ -1984,19 +1990,19 @@ __device__ __noinline__ bool tile_open(uint32_t gt, const uint8_t *__restrict__ 
 }
 
 // Checks a decoded tile's end (the whole CTA): `how` is ct_decode's.
-__device__ __noinline__ void tile_close(int how, const uint8_t *__restrict__ comp, const uint64_t *__restrict__ comp_off,
-                                        int nblk, const uint8_t *__restrict__ ws, int32_t *__restrict__ status) {
+__device__ __noinline__ void tile_close(int how, int nblk, const uint8_t *__restrict__ ws, int32_t *__restrict__ status) {
     CtaTile &S = smem_item<CtaTile>();
     const int t = threadIdx.x, b = S.job.b;
     const uint32_t V = S.job.V, k = S.job.k, ntile = dec_ws(const_cast<uint8_t *>(ws), nblk).blk_ntile[b];
     bool bad = how == kTileBad;
     if (!bad && (uint32_t)t < V) {
-        const TileTabs TT = tile_tabs(ws, nblk, b, comp + comp_off[b], V);
-        const uint32_t nvv = __ldg(TT.nv + t), bpe = max(1u, ch_flat_d(S.ch[t])), s0 = TT.nsrc[3 * t];
         // the chunks must end exactly at the tile's end cursors
-        if (how == kTileChunked && S.pos[t] != s0 + tile_cursor(TT, V, k + 1, ntile, t, S.job.P1, nvv) * bpe) bad = true;
-        // the last tile checks the pad bits of every body
-        if (k + 1 == ntile && pad_bad(S.job.src, s0, nvv * bpe)) bad = true;
+        if (how == kTileChunked && S.pos[t] != S.end[t]) bad = true;
+        // the last tile checks the pad bits of every body (its end cursors are the bodies' ends)
+        if (k + 1 == ntile) {
+            const uint32_t nb = __ldg(reinterpret_cast<const uint32_t *>(S.job.src.rec + kNvOff) + t) * max(1u, ch_flat_d(S.ch[t]));
+            if (pad_bad(S.job.src, S.end[t] - nb, nb)) bad = true;
+        }
     }
     if (__syncthreads_or(bad) && t == 0) status[b] = PIVCO_ERR_CORRUPT;
 }
@@ -2276,7 +2282,7 @@ __global__ void __launch_bounds__(kDecThreads, kTileCtas) decode_kernel(const ui
         __syncthreads();
         if (it >= total_tiles) break;
         if (tile_open(it, comp, comp_off, nblk, out, out_off, ws, ws_bytes, status))
-            tile_close(ct_decode(), comp, comp_off, nblk, ws, status);
+            tile_close(ct_decode(), nblk, ws, status);
     }
 }
 
@@ -2422,7 +2428,7 @@ __device__ __noinline__ bool block_open(const BatchQueue &q, int b) {
                 (bpe > 1 && (chv & 0xFFu) + (1u << bpe) > 256u))
                 bad = true;
             S.pos[t] = s0;
-            S.src0[t] = s0;
+            S.end[t] = s0 + nvv * bpe;
             S.dem[t] = nvv;
             S.ch[t] = chv;
         }
@@ -2470,7 +2476,7 @@ __device__ __noinline__ void block_close(const BatchQueue &q, int b, int how) {
         // the chunks must end exactly at the bodies' ends; pad bits are zero
         const uint32_t nb = __ldg(reinterpret_cast<const uint32_t *>(S.job.src.rec + kNvOff) + t) *
                             max(1u, ch_flat_d(S.ch[t]));
-        bad = pad_bad(S.job.src, S.src0[t], nb) || (how == kTileChunked && S.pos[t] != S.src0[t] + nb);
+        bad = pad_bad(S.job.src, S.end[t] - nb, nb) || (how == kTileChunked && S.pos[t] != S.end[t]);
     }
     // (decoded: whatever another CTA that gave up has marked in the meantime)
     if (__syncthreads_or(bad)) {
@@ -2647,7 +2653,7 @@ __global__ void __launch_bounds__(kDecThreads, kTileCtas) decode_batch_kernel(co
         const int r = batch_item(q, item, A);
         if (r == kItemTile || r == kItemBlock) {
             const int how = ct_decode();
-            if (r == kItemTile) tile_close(how, q.comp, q.comp_off, nblk, q.ws, q.status);
+            if (r == kItemTile) tile_close(how, nblk, q.ws, q.status);
             else block_close(q, (int)item, how);
             __syncthreads();
         } else if (r != kItemDone) {
@@ -2748,7 +2754,7 @@ __global__ void __launch_bounds__(kDecThreads, kTileCtas) serve_loop_kernel(Serv
         int res = batch_item(q, item, A);
         if (res == kItemTile || res == kItemBlock) {
             const int how = ct_decode();
-            if (res == kItemTile) tile_close(how, q.comp, q.comp_off, q.nblk, q.ws, q.status);
+            if (res == kItemTile) tile_close(how, q.nblk, q.ws, q.status);
             else block_close(q, (int)item, how);
             __syncthreads();
             res = kItemDone;
