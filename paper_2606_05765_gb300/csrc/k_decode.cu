@@ -2353,24 +2353,28 @@ struct BatchQueue {
     uint64_t ws_bytes;
     int32_t *status;
     int nblk;
+    bool wide;                  // the form of its queue (wide_batch)
 };
 
 // the wait bound of a batch's queue (workspace header)
 __device__ inline uint64_t wait_bound(const BatchQueue &q) { return reinterpret_cast<const uint64_t *>(q.ws)[7]; }
 
-// Plans by warps, then the blocks' own items: for batches of more blocks than
+// Plans by warps, then the blocks' own items (a wide batch): for more blocks than
 // the launch has CTAs, where the plans' instructions count (4096 blocks of
 // 64 KiB: 150 us of CTA plans, 50 us of warp plans; the line stands where the
 // second wave begins: 862 blocks decode in 166 us by warp plans, 185 by CTA
 // plans); else one item plans and decodes a block, its decode starting 7 us
-// after the item (a warp plan takes 25 us).
-__device__ inline bool batch_wide(const BatchQueue &q) { return (uint32_t)q.nblk > gridDim.x; }
+// after the item (a warp plan takes 25 us).  Decided once per batch: the items of
+// a served request are taken by several launches, which need not have the same
+// number of CTAs (the tuning may change between them), so its form goes with
+// the request.
+__host__ __device__ inline bool wide_batch(int nblk, int ctas) { return nblk > ctas; }
 __device__ inline uint32_t batch_nplan(const BatchQueue &q) {
-    return batch_wide(q) ? (uint32_t)((q.nblk + kDecWarps - 1) / kDecWarps) : 0u;
+    return q.wide ? (uint32_t)((q.nblk + kDecWarps - 1) / kDecWarps) : 0u;
 }
 __device__ inline uint32_t batch_items_blocks(const BatchQueue &q) { return batch_nplan(q) + (uint32_t)q.nblk; }
 // plans to wait for (header word 10 counts them)
-__device__ inline uint32_t batch_plans(const BatchQueue &q) { return batch_wide(q) ? batch_nplan(q) : (uint32_t)q.nblk; }
+__device__ inline uint32_t batch_plans(const BatchQueue &q) { return q.wide ? batch_nplan(q) : (uint32_t)q.nblk; }
 
 // Items of each stage once all plans are done (header written by the last
 // plan; word 12 counts the blocks whose tiles are still to be decoded).
@@ -2499,7 +2503,7 @@ __device__ __noinline__ int batch_item(const BatchQueue &q, uint32_t item, const
     const int nblk = q.nblk;
     uint32_t *hdr = reinterpret_cast<uint32_t *>(q.ws);
     const DecWs W = dec_ws(q.ws, nblk);
-    if (!batch_wide(q)) {
+    if (!q.wide) {
         if (item < (uint32_t)nblk) {
             return block_open(q, (int)item) ? kItemBlock : kItemDone;
         }
@@ -2642,7 +2646,7 @@ __global__ void __launch_bounds__(kDecThreads, kTileCtas) decode_batch_kernel(co
     extern __shared__ __align__(128) uint8_t smem_raw[];
     BatchSmem &B = *reinterpret_cast<BatchSmem *>(smem_raw);
     __shared__ uint32_t s_item;
-    const BatchQueue q{comp, comp_off, out, out_off, ws, ws_bytes, status, nblk};
+    const BatchQueue q{comp, comp_off, out, out_off, ws, ws_bytes, status, nblk, wide_batch(nblk, (int)gridDim.x)};
     uint32_t *hdr = reinterpret_cast<uint32_t *>(ws);
     sel_init(B.sel);
     for (;;) {
@@ -2750,7 +2754,7 @@ __global__ void __launch_bounds__(kDecThreads, kTileCtas) serve_loop_kernel(Serv
             if (t == 0) __nanosleep(1000);
             continue;
         }
-        const BatchQueue q{D.comp, D.comp_off, D.out, D.out_off, D.ws, D.ws_bytes, D.status, D.nblk};
+        const BatchQueue q{D.comp, D.comp_off, D.out, D.out_off, D.ws, D.ws_bytes, D.status, (int)D.nblk, D.wide != 0};
         int res = batch_item(q, item, A);
         if (res == kItemTile || res == kItemBlock) {
             const int how = ct_decode();
@@ -3008,6 +3012,10 @@ cudaError_t launch_decode_merge(const uint8_t *comp, const uint64_t *comp_off, i
         comp, comp_off, nblk, out, out_off, ws, ws_bytes, status);
     count_launches(1);
     return cudaGetLastError();
+}
+
+bool serve_wide(int nblk) {
+    return wide_batch(nblk, merge_grid((const void *)serve_loop_kernel, (int)sizeof(BatchSmem)));
 }
 
 cudaError_t launch_serve_loop(ServeCtl *ctl, const ServeDesc *ring, ServeFlags *flags, uint64_t idle_ns,

@@ -550,7 +550,8 @@ struct ServeDesc {                          // one published request (device mem
     uint8_t *ws;
     uint64_t ws_bytes;
     int32_t *status;
-    int32_t nblk;
+    uint32_t nblk : 31;
+    uint32_t wide : 1;                      // the form of its queue (wide_batch), for every launch that takes its items
     uint32_t seq;
 };
 static_assert(sizeof(ServeDesc) == 64, "ring entry layout");
@@ -565,6 +566,7 @@ struct ServeFlags {                         // pinned host memory mapped into th
     uint32_t done[kServeRing];              // seq + 1 once request seq is decoded (device writes)
     int32_t worst[kServeRing];              // its first non-OK block status, else 0 (device writes)
 };
+bool serve_wide(int nblk);   // the form of a request's queue under the tuning of this moment
 cudaError_t launch_serve_loop(ServeCtl *ctl, const ServeDesc *ring, ServeFlags *flags, uint64_t idle_ns,
                               uint64_t life_ns, cudaStream_t st);
 size_t decode_ws_bound(const uint8_t *comp, const uint64_t *comp_off, int nblk, const DecTuning &tu);

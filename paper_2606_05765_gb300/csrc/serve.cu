@@ -184,7 +184,8 @@ struct pivco_server {
             dsc.ws = d_ws;
             dsc.ws_bytes = r->ws_bytes;
             dsc.status = d_st;
-            dsc.nblk = r->nblk;
+            dsc.nblk = (uint32_t)r->nblk;
+            dsc.wide = pv::serve_wide(r->nblk);
             dsc.seq = (uint32_t)r->seq;
             if (e == cudaSuccess) e = cudaMemcpyAsync(ring_d + slot, &dsc, sizeof(dsc), cudaMemcpyHostToDevice, s_in);
             r->ev_in = get_event();
