@@ -447,6 +447,8 @@ __device__ inline void enc_part(EncSmem &S, const uint8_t *src, uint32_t C, cons
             }
             par ^= 1u;
         }
+        // (carry: all the root's ones; too few symbols for a child would leave its span as the buffer was)
+        if ((i1 && carry != dem1) || (i0 && C - carry != dem0)) bad = true;
         if (code && (i0 || i1)) {
             // the kept symbols are input bytes still: their code indices
             __syncthreads();
@@ -527,8 +529,11 @@ __device__ inline void enc_part(EncSmem &S, const uint8_t *src, uint32_t C, cons
                 const uint32_t r1 = (ex + inc - ps - S.fw[v]) & 0xFFFFu, kk = kGrp * q, vl = min(32u, left);
                 const uint32_t chv = S.ch[v], c0 = chv & 0xFFFFu, c1 = chv >> 16;
                 const bool i0 = left && !(c0 & 0x8000u), i1 = left && !(c1 & 0x8000u);
-                const bool over = (i1 && r1 + pc > S.dem[c1 & 0xFFu]) || (i0 && kk + vl - r1 - pc > S.dem[c0 & 0xFFu]);
-                if (over) bad = true;
+                const uint32_t n0 = kk + vl - r1 - pc, n1 = r1 + pc;
+                const uint32_t d0 = i0 ? S.dem[c0 & 0xFFu] : n0, d1 = i1 ? S.dem[c1 & 0xFFu] : n1;
+                const bool over = n0 > d0 || n1 > d1;
+                // the node's last group: its children have got exactly what they count
+                if (over || (left <= 32 && (n0 != d0 || n1 != d1))) bad = true;
                 EncGrp G;
                 G.w = w;
                 G.a = over ? 0u : (((i0 ? (uint32_t)S.sp[c0 & 0xFFu] : 0u) + kk - r1) & 0xFFFFu) |
