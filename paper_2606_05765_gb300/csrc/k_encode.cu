@@ -877,9 +877,10 @@ __global__ void __launch_bounds__(kEncThreads) encode_reset_kernel(const uint64_
 // and finding each entry's place, quadratic in the list, costs more.)
 constexpr uint32_t kEncSortMax = 2048;
 
-// Entry i of the list goes to its place by size (whole CTA, before the chunk kernel).
+// Entry i of the list goes to its place by size (whole CTA); counted in
+// list_placed, whose release the chunk kernel acquires.
 __device__ inline void enc_list_place(uint32_t i, uint32_t len, const uint64_t *__restrict__ blk_off,
-                                      const BlockLayout *layout) {
+                                      BlockLayout *layout) {
     auto size_of = [&](uint32_t j) {
         const uint32_t b = layout_of(layout, (int)j)->list_entry;
         return blk_off[b + 1] - blk_off[b];
@@ -896,8 +897,8 @@ __device__ inline void enc_list_place(uint32_t i, uint32_t len, const uint64_t *
         place += __syncthreads_count(before);
     }
     if (threadIdx.x == 0) {
-        __stcg(&const_cast<BlockLayout *>(layout_of(layout, place))->list_sorted, layout_of(layout, (int)i)->list_entry);
-        __threadfence();
+        __stcg(&layout_of(layout, place)->list_sorted, layout_of(layout, (int)i)->list_entry);
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&layout->list_placed) : "memory");
     }
     __syncthreads();
 }
@@ -906,7 +907,7 @@ __device__ inline void enc_list_place(uint32_t i, uint32_t len, const uint64_t *
 // kernel).
 __global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm) encode_kernel(const uint8_t *__restrict__ in,
                                                                             const uint64_t *__restrict__ blk_off,
-                                                                            const BlockLayout *__restrict__ layout,
+                                                                            BlockLayout *layout,
                                                                             const uint32_t *__restrict__ chunk_hist,
                                                                             uint8_t *__restrict__ out,
                                                                             const uint64_t *__restrict__ out_off,
@@ -935,12 +936,38 @@ __global__ void __launch_bounds__(kEncThreads, kEncCtasPerSm) encode_chunks_kern
                                                                               uint8_t *__restrict__ out,
                                                                               const uint64_t *__restrict__ out_off,
                                                                               uint64_t *__restrict__ rec_bytes,
-                                                                              int32_t *__restrict__ status) {
+                                                                              int32_t *__restrict__ status, bool early,
+                                                                              uint64_t limit_ns) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     EncSmem &S = *reinterpret_cast<EncSmem *>(smem_raw);
     __shared__ uint32_t s_tk;
-    // (the list and its order are complete: all of encode_kernel's CTAs are past writing them)
-    const uint32_t len = __ldcg(&layout->list_len), chunks = len * kEncChunks;
+    // Of what encode_kernel writes, only the list's order is read here.  Started early, this kernel runs once all
+    // of its CTAs are past the trigger, which they reach after placing their entries; the trigger does not order
+    // those writes, their count does.  (The list itself and all else was there before encode_kernel started.)
+    const uint32_t len = __ldcg(&layout->list_len);
+    if (early && len && len <= kEncSortMax) {
+        if (threadIdx.x == 0) {
+            const uint64_t t0 = globaltimer_ns();
+            uint32_t v;
+            for (;;) {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&layout->list_placed) : "memory");
+                if (v >= len || globaltimer_ns() - t0 > limit_ns) break;
+                __nanosleep(64);
+            }
+            s_tk = v;
+        }
+        __syncthreads();
+        if (s_tk < len) {   // the wait ran out: the list's blocks are given up
+            for (uint32_t i = threadIdx.x; i < len; i += kEncThreads) {
+                const uint32_t b = __ldcg(&layout_of(layout, (int)i)->list_entry);
+                atomicExch(&status[b], PIVCO_ERR_TIMEOUT);
+                rec_bytes[b] = 0;
+            }
+            if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+            return;
+        }
+    }
+    const uint32_t chunks = len * kEncChunks;
     const uint32_t shares = min(kEncShares, max(1u, gridDim.x / max(1u, chunks))), items = chunks * shares;
     // an item each: by the CTA's number, which the launch deals out over the SMs (tickets taken in the order
     // of arrival put four of the 64 shares of one block on some SMs and none on others: 85 us, 52 spread).
@@ -978,7 +1005,7 @@ cudaError_t launch_encode(const uint8_t *in, const uint64_t *blk_off, int nblk, 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // the work list of big blocks: emptied, then filled by the reset pass
-    e = cudaMemsetAsync(&layout->list_len, 0, 2 * sizeof(uint32_t), st);
+    e = cudaMemsetAsync(&layout->list_len, 0, 3 * sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
     if (chunk_hist) {
         // (several CTAs per block when the blocks alone do not fill the chip: one block of 1 MiB 17 us by one CTA,
@@ -1005,8 +1032,10 @@ cudaError_t launch_encode(const uint8_t *in, const uint64_t *blk_off, int nblk, 
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
-        cfg.numAttrs = nblk > sms ? 1 : 0;
-        e = cudaLaunchKernelEx(&cfg, encode_chunks_kernel, in, blk_off, layout, chunk_hist, out, out_off, rec_bytes, status);
+        const bool early = nblk > sms;
+        cfg.numAttrs = early ? 1 : 0;
+        e = cudaLaunchKernelEx(&cfg, encode_chunks_kernel, in, blk_off, layout, chunk_hist, out, out_off, rec_bytes, status,
+                               early, wait_limit_ns());
         if (e != cudaSuccess) return e;
         count_launches(1);
     }

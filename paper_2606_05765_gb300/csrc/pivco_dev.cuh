@@ -97,12 +97,14 @@ struct BlockLayout {
     // scratch of the chunked encoder (the work list of big blocks; written
     // by the encode call, not by the plan): entry i of the list lives in
     // block i's layout (with the list's entry that comes i-th by size), its
-    // length and the chunk ticket in block 0's
+    // length, the chunk ticket and the entries placed by size in block 0's
     uint32_t list_entry;
-    uint32_t list_len;
+    uint32_t list_len;         // (these three are set to 0 together)
     uint32_t list_ticket;
+    uint32_t list_placed;
     uint32_t list_sorted;
 };
+static_assert(offsetof(BlockLayout, list_placed) == offsetof(BlockLayout, list_len) + 8, "one run");
 static_assert(offsetof(BlockLayout, ci) % 16 == 0 && offsetof(BlockLayout, nhi1) + 256 == offsetof(BlockLayout, ci) + 768,
               "the canonical tables are one 16-byte aligned run");
 static_assert(sizeof(BlockLayout) <= 8192, "layout too large");
