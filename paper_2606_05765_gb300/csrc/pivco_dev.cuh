@@ -76,7 +76,8 @@ struct BlockLayout {
     uint8_t depth_first[17];   // first node id at depth d (breadth-first); [d+1]-[d] = count
     uint8_t big;               // the levels of the whole block do not fit the encoder's buffers
     uint8_t pad1[2];
-    uint32_t part;             // symbols of an encoder part whose levels fit its buffers with room to spare
+    uint32_t part;             // symbols of an encoder part: the whole block where its levels fit the buffers, else
+                               // as many as fit with room to spare
     uint8_t pad4b[8];
     uint16_t tree_a[17];       // leaf-covered prefix count at depth d (TreeShape::a)
     uint16_t pad2[15];
