@@ -384,7 +384,25 @@ cudaError_t launch_code_lengths(const uint32_t *hist, int nblk, int max_len, uin
 struct SelectParams {
     pivco_params p;
     int32_t fseh_q16[50];
+    uint32_t split;             // blocks of at least this size are split over several CTAs
 };
+
+// The parameters for a batch of nblk blocks.  It splits its blocks when the
+// chunks of all of them run at once: 20 to 76 blocks of 100000 symbols, 90 us
+// by one CTA each, 70 to 78 by chunks (65536: 76 and 66 to 70; 16384 to 40000:
+// the same within 5 %); 100 blocks of them 91 and 105, 152 of 40000 69 and 94.
+static SelectParams select_params(const pivco_params &p, int nblk, int &sms) {
+    SelectParams sp;
+    sp.p = p;
+    const AnsTables &T = host_ans_tables();
+    for (int i = 0; i < 50; i++) sp.fseh_q16[i] = T.fseh_q16[i];
+    int dev = 0;
+    sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sp.split = (int64_t)nblk * kEncChunks <= (int64_t)sms * kEncCtasPerSm ? kEncSplitSize : 0xFFFFFFFFu;
+    return sp;
+}
 
 // Sec. 5.2: selected when ceil(n/8) >= min bytes, skew > num/den and
 // (depth + fse_H) / (depth + 1) < ratio.  Table t = round(100 * skew) in
@@ -420,7 +438,7 @@ struct LaySmem {
 
 // Layout of block b from its histogram h and lengths lens (both shared, 256)
 // by one CTA of 256 threads: written to layout[b], rec_bound[b], status[b].
-__device__ inline void build_layout_block(int b, int nblk, const uint32_t *h, const uint8_t *lens, const SelectParams &sp,
+__device__ inline void build_layout_block(int b, const uint32_t *h, const uint8_t *lens, const SelectParams &sp,
                                           LaySmem &Y, BlockLayout *__restrict__ layout,
                                           uint64_t *__restrict__ rec_bound, int32_t *__restrict__ status) {
     BlockLayout &L = Y.L;
@@ -578,9 +596,8 @@ __device__ inline void build_layout_block(int b, int nblk, const uint32_t *h, co
                 // a big block is coded chunk by chunk by several CTAs: some
                 // level (depth >= 1) of the whole block does not fit an
                 // encoder level buffer (spans of whole 16-byte units), or
-                // the batch has too few blocks to fill the chip with one CTA
-                // each
-                if (t == 0 && nblk <= (int)kEncFewBlocks && n >= kEncFewSize && maxd > 1) L.big = 1;
+                // the batch has few blocks (select_params)
+                if (t == 0 && n >= sp.split && maxd > 1) L.big = 1;
                 float part = (float)n;   // (1024 symbols and more: its rounding is far below the 10 % to spare)
                 // only a level that does not fit cuts the block into parts: the others' spans hold any part of it
                 for (int d = 1 + (t >> 5); d < maxd; d += kLayThreads / 32) {   // a warp per level
@@ -667,7 +684,7 @@ __global__ void __launch_bounds__(kLayThreads) build_layout_kernel(const uint32_
     const int b = blockIdx.x, t = threadIdx.x;
     h[t] = hist[(size_t)b * 256 + t];
     lens[t] = lens_in[(size_t)b * 256 + t];
-    build_layout_block(b, gridDim.x, h, lens, sp, Y, layout, rec_bound, status);
+    build_layout_block(b, h, lens, sp, Y, layout, rec_bound, status);
 }
 
 // The encoder's planning in one launch, one CTA per block: chunk histograms,
@@ -691,14 +708,14 @@ struct PlanSmem {
 // 125 us of the plan: there the extra CTAs' coming and going takes what they save.)
 constexpr uint32_t kPlanWide = 32768;
 
-__device__ inline void plan_rest(int b, int nblk, int max_len, const SelectParams &sp, PlanSmem &P,
+__device__ inline void plan_rest(int b, int max_len, const SelectParams &sp, PlanSmem &P,
                                  uint8_t *__restrict__ lens_out, BlockLayout *__restrict__ layout,
                                  uint64_t *__restrict__ rec_bound, int32_t *__restrict__ status) {
     __syncthreads();
     code_lengths_block(P.h, max_len, P.u.cl, P.lens);   // (its status is the layout's too)
     lens_out[(size_t)b * 256 + threadIdx.x] = P.lens[threadIdx.x];
     __syncthreads();
-    build_layout_block(b, nblk, P.h, P.lens, sp, P.u.lay, layout, rec_bound, status);
+    build_layout_block(b, P.h, P.lens, sp, P.u.lay, layout, rec_bound, status);
 }
 
 static_assert(kHistThreads == kPmThreads && kPmThreads == kLayThreads, "one CTA shape for the three steps");
@@ -710,7 +727,7 @@ __global__ void __launch_bounds__(kHistThreads, 8) block_plan_kernel(
     int32_t *__restrict__ status) {
     __shared__ PlanSmem P;
     histogram_chunks_block(blockIdx.x, in, blk_off, hist, chunk_hist, P.u.wh, P.h);
-    plan_rest(blockIdx.x, gridDim.x, max_len, sp, P, lens_out, layout, rec_bound, status);
+    plan_rest(blockIdx.x, max_len, sp, P, lens_out, layout, rec_bound, status);
 }
 
 __global__ void __cluster_dims__(kEncChunks, 1, 1) __launch_bounds__(kHistThreads)
@@ -736,20 +753,15 @@ __global__ void __cluster_dims__(kEncChunks, 1, 1) __launch_bounds__(kHistThread
         if (c) return;
         histogram_chunks_block(b, in, blk_off, hist, chunk_hist, P.u.wh, P.h);
     }
-    plan_rest(b, gridDim.x / kEncChunks, max_len, sp, P, lens_out, layout, rec_bound, status);
+    plan_rest(b, max_len, sp, P, lens_out, layout, rec_bound, status);
 }
 
 cudaError_t launch_block_plan(const uint8_t *in, const uint64_t *blk_off, int nblk, const pivco_params &p,
                               uint32_t *hist, uint32_t *chunk_hist, uint8_t *lens, BlockLayout *layout,
                               uint64_t *rec_bound, int32_t *status, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
-    SelectParams sp;
-    sp.p = p;
-    const AnsTables &T = host_ans_tables();
-    for (int i = 0; i < 50; i++) sp.fseh_q16[i] = T.fseh_q16[i];
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms;
+    const SelectParams sp = select_params(p, nblk, sms);
     if (nblk * (int)kEncChunks <= sms)
         block_plan_cluster_kernel<<<nblk * (int)kEncChunks, kHistThreads, 0, st>>>(in, blk_off, p.max_len, sp, hist, chunk_hist,
                                                                                     lens, layout, rec_bound, status);
@@ -763,10 +775,8 @@ cudaError_t launch_block_plan(const uint8_t *in, const uint64_t *blk_off, int nb
 cudaError_t launch_build_layout(const uint32_t *hist, const uint8_t *lens, int nblk, const pivco_params &p,
                                 BlockLayout *layout, uint64_t *rec_bound, int32_t *status, cudaStream_t st) {
     if (nblk <= 0) return cudaSuccess;
-    SelectParams sp;
-    sp.p = p;
-    const AnsTables &T = host_ans_tables();
-    for (int i = 0; i < 50; i++) sp.fseh_q16[i] = T.fseh_q16[i];
+    int sms;
+    const SelectParams sp = select_params(p, nblk, sms);
     build_layout_kernel<<<nblk, kLayThreads, 0, st>>>(hist, lens, sp, layout, rec_bound, status);
     count_launches(1);
     return cudaGetLastError();

@@ -36,7 +36,6 @@ namespace pv {
 
 constexpr int kEncThreads = 256;
 constexpr int kEncWarps = kEncThreads / 32;
-constexpr int kEncCtasPerSm = 4;
 static_assert(kEncWarps == kLvlWarps, "the level tables are laid out by all warps");
 
 struct __align__(16) EncSmem {

@@ -74,7 +74,7 @@ struct BlockLayout {
     uint8_t status;        // PIVCO_* of layout construction
     uint8_t flat;          // regrouped tree with flat subtrees (record tag PVC2)
     uint8_t depth_first[17];   // first node id at depth d (breadth-first); [d+1]-[d] = count
-    uint8_t big;               // the levels of the whole block do not fit the encoder's buffers
+    uint8_t big;               // coded by several CTAs: its levels do not fit the encoder's buffers, or the batch is small
     uint8_t pad1[2];
     uint32_t part;             // symbols of an encoder part: the whole block where its levels fit the buffers, else
                                // as many as fit with room to spare
@@ -442,12 +442,10 @@ inline int div_up(long long a, long long b) { return (int)((a + b - 1) / b); }
 // counts each chunk on its own; the chunks of a big block are coded by
 // several CTAs.
 constexpr uint32_t kEncChunks = 8;
-constexpr int kEBuf = 22016;         // symbols per encoder level buffer (4 CTAs per SM)
+constexpr int kEncCtasPerSm = 4;
+constexpr int kEBuf = 22016;         // symbols per encoder level buffer (kEncCtasPerSm CTAs per SM)
 constexpr uint32_t kEncShares = 8;   // shares of a chunk at most
-// Batches of at most this many blocks split their blocks of at least this
-// size over several CTAs (26 blocks of 39-79 KB, plan to ANS: 162 us by one CTA
-// each, 124 us by chunks)
-constexpr uint32_t kEncFewBlocks = 152, kEncFewSize = 16384;
+constexpr uint32_t kEncSplitSize = 16384;   // batches of few blocks split theirs of at least this size over several CTAs
 constexpr uint32_t kEncMinChunk = 4096;
 __host__ __device__ inline uint32_t enc_nchunks(uint64_t n) {
     const uint64_t c = n / kEncMinChunk;
