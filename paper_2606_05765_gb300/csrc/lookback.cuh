@@ -68,12 +68,22 @@ __device__ inline uint64_t lookback_exclusive(uint64_t *states, int tile, uint64
 // the tile's other work; lookback2_cta waits for the predecessors' (bounded),
 // publishes the inclusive prefixes and returns the exclusive ones in every
 // thread.  Returns true when the wait ran out or a poisoned prefix was met.
+// A state holds all that is taken from it, so its loads and stores order
+// nothing else.
 constexpr int kLbThreads = 256;
 constexpr int kLbWarps = kLbThreads / 32;
+__device__ inline void lb2_store(uint64_t *p, uint64_t v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ inline uint64_t lb2_load(const uint64_t *p) {
+    uint64_t v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ inline void lb2_publish(uint64_t *states_a, uint64_t *states_b, int tile, uint64_t agg_a, uint64_t agg_b) {
     const uint64_t f = tile == 0 ? kLbFlagInc : kLbFlagAgg;
-    lb_store(&states_a[tile], f | (agg_a & kLbValMask));
-    lb_store(&states_b[tile], f | (agg_b & kLbValMask));
+    lb2_store(&states_a[tile], f | (agg_a & kLbValMask));
+    lb2_store(&states_b[tile], f | (agg_b & kLbValMask));
 }
 __device__ inline bool lookback2_cta(uint64_t *states_a, uint64_t *states_b, int tile, uint64_t agg_a, uint64_t agg_b,
                                      uint64_t &excl_a, uint64_t &excl_b, uint64_t limit_ns, uint32_t (*mins)[4],
@@ -87,8 +97,8 @@ __device__ inline bool lookback2_cta(uint64_t *states_a, uint64_t *states_b, int
     unsigned ns = 32;
     for (;;) {
         const int k = j - t;
-        const uint64_t va = k >= 0 ? lb_load(&states_a[k]) : kLbFlagInc;   // before tile 0: an inclusive zero
-        const uint64_t vb = k >= 0 ? lb_load(&states_b[k]) : kLbFlagInc;
+        const uint64_t va = k >= 0 ? lb2_load(&states_a[k]) : kLbFlagInc;   // before tile 0: an inclusive zero
+        const uint64_t vb = k >= 0 ? lb2_load(&states_b[k]) : kLbFlagInc;
         const uint64_t fa = va & (kLbFlagAgg | kLbFlagInc), fb = vb & (kLbFlagAgg | kLbFlagInc);
         // both chains are published one right after the other: a state counts once they agree
         const bool inc = fa == kLbFlagInc && fb == kLbFlagInc, agg = fa == kLbFlagAgg && fb == kLbFlagAgg;
@@ -131,8 +141,8 @@ __device__ inline bool lookback2_cta(uint64_t *states_a, uint64_t *states_b, int
     __syncthreads();
     if (t == 0) {
         const uint64_t p = bad ? kLbPoison : 0ull;
-        lb_store(&states_a[tile], kLbFlagInc | p | ((excl_a + agg_a) & kLbValMask));
-        lb_store(&states_b[tile], kLbFlagInc | p | ((excl_b + agg_b) & kLbValMask));
+        lb2_store(&states_a[tile], kLbFlagInc | p | ((excl_a + agg_a) & kLbValMask));
+        lb2_store(&states_b[tile], kLbFlagInc | p | ((excl_b + agg_b) & kLbValMask));
     }
     return bad;
 }
