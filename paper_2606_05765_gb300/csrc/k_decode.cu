@@ -1662,7 +1662,7 @@ __device__ __forceinline__ void ct_root(CtaTile &S, const TileSrc &src, uint8_t 
     BitLd nx{0u, 0u, 0u};
     if (kWin * m * warp + kGrp * lane < dv) nx = tile_ld(src, pos, kWin * m * warp + kGrp * lane);
     for (uint32_t s = warp; s * m < nwin; s += kTileWarps) {
-        uint32_t carry = S.strip[s];
+        uint32_t carry = HL || HR ? S.strip[s] : 0u;
         const uint32_t iend = min(nwin, (s + 1) * m);
         for (uint32_t i = s * m; i < iend; i++) {
             const uint32_t w = root_mask(tile_word(nx), kWin * i + kGrp * lane, dv);
@@ -1835,10 +1835,12 @@ __device__ __forceinline__ int ct_decode() {
         }
         bool ok = true;
         for (int d = S.maxd - 1; d >= 1; d--) ok = ct_level(S, src, d, sel, par) && ok;
-        if (!ch_flat_d(S.ch[0])) ct_count_root(S, src);   // (its barriers also end the level below)
+        // (a flat root, or one of two leaves, needs no ranks and has no level below, which the barriers here also end)
+        const bool ranked = (S.ch[0] & 0x80008000u) != 0x80008000u;
+        if (ranked) ct_count_root(S, src);
         if (reinterpret_cast<uintptr_t>(dst + P) & 7) ct_root_any<true>(S, src, dst + P, sel);
         else ct_root_any<false>(S, src, dst + P, sel);
-        if (!ch_flat_d(S.ch[0])) ok = children_ok(S, S.ch[0], S.dem[0], S.rtot) && ok;
+        if (ranked) ok = children_ok(S, S.ch[0], S.dem[0], S.rtot) && ok;
         if (__syncthreads_or(!ok)) return kTileBad;
         if ((uint32_t)t < V) S.pos[t] += S.dem[t] * max(1u, ch_flat_d(S.ch[t]));
         __syncthreads();
