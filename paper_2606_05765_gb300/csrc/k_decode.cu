@@ -2017,11 +2017,12 @@ __device__ __noinline__ void tile_close(int how, int nblk, const uint8_t *__rest
 //                  each), counted from the node's start or the start of the
 //                  share the entry lies in, whichever is later
 //   cur[k V + v]   node v's bitmap cursor at tile boundary k (k = 1 ..
-//                  ntile - 1, v >= 1); cur[s V], s < shares: share s's tail,
-//                  the ones of its last node within it
-// The superblocks of a block are cut into at most min(ntile, 128) shares of
-// 2^s entries, so that building them is work of as many warps as the block
-// has tiles, in two steps:
+//                  ntile - 1, v >= 1); the other places (k = 0, k = ntile,
+//                  v = 0) hold the shares' tails: the ones of a share's last
+//                  node within it
+// The superblocks of a block are cut into at most 128 shares of 2^s entries,
+// `ways` times as many as the block has tiles at most (1 in batches of many
+// tiles, where the chip is full either way), in two steps:
 //   shares    a warp counts the superblocks of one share
 //   cursors   a warp takes one tile boundary: the root's cursor is k T;
 //             top-down, a child's cursor is the parent's rank0 / rank1 there
@@ -2034,11 +2035,18 @@ __device__ __noinline__ void tile_close(int how, int nblk, const uint8_t *__rest
 // 29 us.
 // ---------------------------------------------------------------------------
 constexpr uint32_t kDirShares = 128;   // shares of a block at most
-constexpr uint32_t kDirShareMin = 10;  // log2 of the fewest entries of a share (but for the block's last)
+constexpr uint32_t kDirShareMin = 10;  // log2 of the fewest entries of a share (but for the block's last) ...
+constexpr uint32_t kDirShareFew = 7;   // ... in batches of few tiles: one step of dir_share_count
+constexpr uint32_t kDirTarget = 4864;  // about as many shares as warps of the pass run at once (four CTAs an SM)
+constexpr uint32_t kDirWays = 8;
 
-__device__ inline uint32_t dir_share_log(uint32_t ent, uint32_t ntile) {
-    const uint32_t most = min(ntile, kDirShares);
-    uint32_t s = kDirShareMin;
+// Shares for each of the batch's tiles (a function of the tiles alone: the
+// items of a served request are numbered by it).
+__device__ inline uint32_t dir_ways(uint32_t tiles) { return max(1u, min(kDirWays, kDirTarget / max(1u, tiles))); }
+
+__device__ inline uint32_t dir_share_log(uint32_t ent, uint32_t V, uint32_t ntile, uint32_t ways) {
+    const uint32_t most = ways == 1 ? min(ntile, kDirShares) : min(min(ntile * ways, kDirShares), 2 * V + ntile - 1);
+    uint32_t s = ways == 1 ? kDirShareMin : kDirShareFew;
     while (s < 31 && (ent >> s) + ((ent & ((1u << s) - 1u)) != 0) > most) s++;
     return s;
 }
@@ -2057,8 +2065,13 @@ struct DirRef {
     uint32_t V, ent, ntile, T, slog, shares;
     uint32_t *dirp, *cur;
     TileSrc src;
+    // where share s's tail is kept: boundary 0's places, the end's, the root's (fewer than 2 V + ntile)
+    __device__ uint32_t *tail(uint32_t s) const {
+        return cur + (s < V ? s : s < 2 * V ? (size_t)ntile * V + (s - V) : (size_t)(s - 2 * V + 1) * V);
+    }
 };
-__device__ inline bool dir_ref(int b, uint32_t k, const uint8_t *__restrict__ comp, const uint64_t *__restrict__ comp_off,
+// (share: k is a share, and there is nothing to do past the last one)
+__device__ inline bool dir_ref(int b, uint32_t k, bool share, const uint8_t *__restrict__ comp, const uint64_t *__restrict__ comp_off,
                                int nblk, uint8_t *__restrict__ ws, uint64_t ws_bytes, int32_t *__restrict__ status,
                                DirWarpSm &M, DirRef &D) {
     const int lane = threadIdx.x & 31;
@@ -2083,8 +2096,9 @@ __device__ inline bool dir_ref(int b, uint32_t k, const uint8_t *__restrict__ co
     }
     D.dirp = reinterpret_cast<uint32_t *>(ws + nbase + ntb);
     D.cur = D.dirp + D.ent;
-    D.slog = dir_share_log(D.ent, D.ntile);
+    D.slog = dir_share_log(D.ent, D.V, D.ntile, dir_ways(reinterpret_cast<const uint32_t *>(ws)[6]));
     D.shares = (D.ent + (1u << D.slog) - 1) >> D.slog;
+    if (share && k >= D.shares) return false;
     const uint64_t sbase = G.scratch + W.blk_scratch[b];
     D.src.rec = rec;
     D.src.rec_bytes = ld_le32(rec);
@@ -2113,6 +2127,7 @@ template <int kW>
 __device__ inline void dir_share_count(const DirRef &D, const DirWarpSm &M, uint32_t k, uint32_t dir_bits) {
     const int lane = threadIdx.x & 31;
     const uint32_t V = D.V;
+    uint32_t *const tail = D.tail(k);
     const uint32_t g0 = k << D.slog, g1 = min(D.ent, g0 + (1u << D.slog));
     const uint32_t le = 0xFFFFFFFFu >> (31 - lane);
     uint32_t vcur = (uint32_t)find_node_d(M.u, 0, (int)V, g0), carry = 0;
@@ -2155,14 +2170,14 @@ __device__ inline void dir_share_count(const DirRef &D, const DirWarpSm &M, uint
                 carry = __shfl_sync(0xffffffffu, ex + pc[r], (int)min(31u, g1 - 1 - (base + 32 * r)));
         }
     }
-    if (lane == 0) D.cur[(size_t)k * V] = carry;
+    if (lane == 0) *tail = carry;
 }
 __device__ __noinline__ void dir_share(int b, uint32_t k, const uint8_t *__restrict__ comp,
                                        const uint64_t *__restrict__ comp_off, int nblk, uint8_t *__restrict__ ws,
                                        uint64_t ws_bytes, int32_t *__restrict__ status) {
     DirWarpSm &M = (&smem_item<DirWarpSm>())[threadIdx.x >> 5];
     DirRef D;
-    if (!dir_ref(b, k, comp, comp_off, nblk, ws, ws_bytes, status, M, D) || k >= D.shares) return;
+    if (!dir_ref(b, k, true, comp, comp_off, nblk, ws, ws_bytes, status, M, D)) return;
     const uint32_t dir_bits = dec_dir_bits(ws);
     if (dir_bits <= 128) dir_share_count<5>(D, M, k, dir_bits);
     else dir_share_count<9>(D, M, k, dir_bits);
@@ -2176,11 +2191,11 @@ __device__ __noinline__ void dir_cursors(int b, uint32_t k, const uint8_t *__res
     const int lane = threadIdx.x & 31;
     DirWarpSm &M = (&smem_item<DirWarpSm>())[threadIdx.x >> 5];
     DirRef D;
-    if (k == 0 || !dir_ref(b, k, comp, comp_off, nblk, ws, ws_bytes, status, M, D) || k >= D.ntile) return;
+    if (k == 0 || !dir_ref(b, k, false, comp, comp_off, nblk, ws, ws_bytes, status, M, D) || k >= D.ntile) return;
     const uint32_t dir_bits = dec_dir_bits(ws), V = D.V;
     uint32_t carry = 0;   // tails of the shares before each share
     for (uint32_t s = 0; s < D.shares; s += 32) {
-        const uint32_t x = s + lane < D.shares ? __ldcg(D.cur + (size_t)(s + lane) * V) : 0u;
+        const uint32_t x = s + lane < D.shares ? __ldcg(D.tail(s + lane)) : 0u;
         const uint32_t inc = warp_inclusive(x);
         if (s + lane < D.shares) M.base[s + lane] = carry + inc - x;
         carry += __shfl_sync(0xffffffffu, inc, 31);
@@ -2224,11 +2239,11 @@ __device__ inline void dir_rebase(int b, uint32_t k, const uint8_t *__restrict__
     const int lane = threadIdx.x & 31;
     DirWarpSm &M = (&smem_item<DirWarpSm>())[threadIdx.x >> 5];
     DirRef D;
-    if (k == 0 || !dir_ref(b, k, comp, comp_off, nblk, ws, ws_bytes, status, M, D) || k >= D.shares) return;
+    if (k == 0 || !dir_ref(b, k, true, comp, comp_off, nblk, ws, ws_bytes, status, M, D)) return;
     const uint32_t g0 = k << D.slog, g1 = min(D.ent, g0 + (1u << D.slog));
     const uint32_t v = (uint32_t)find_node_d(M.u, 0, (int)D.V, g0);
     uint32_t x = 0;
-    for (uint32_t s = (M.u[v] >> D.slog) + lane; s < k; s += 32) x += __ldcg(D.cur + (size_t)s * D.V);
+    for (uint32_t s = (M.u[v] >> D.slog) + lane; s < k; s += 32) x += __ldcg(D.tail(s));
     x = __reduce_add_sync(0xffffffffu, x);
     const uint32_t ge = min(g1, v + 1 < D.V ? M.u[v + 1] : D.ent);
     if (x)
@@ -2239,7 +2254,7 @@ constexpr int kDirSmem = (int)(kSelBytes + sizeof(DirWarpSm) * kDecWarps);   // 
 static_assert(kDirSmem <= 48 * 1024, "no opt-in needed");
 enum : int { kDirShare = 0, kDirCursors = 1, kDirRebase = 2 };
 
-// One step of the directory pass over every tile's share or boundary, one
+// One step of the directory pass over every tile's shares or boundary, one
 // warp each.
 template <int kStep>
 __global__ void __launch_bounds__(kDecThreads) decode_dir_kernel(const uint8_t *__restrict__ comp,
@@ -2248,12 +2263,14 @@ __global__ void __launch_bounds__(kDecThreads) decode_dir_kernel(const uint8_t *
                                                                  int32_t *__restrict__ status) {
     if (abandoned_batch(ws, status, nblk)) return;
     const uint32_t tiles = reinterpret_cast<const uint32_t *>(ws)[6];
-    if (tiles == (uint32_t)nblk && (kStep != kDirShare || !dec_all_dirs(ws))) return;   // one tile each
+    if (tiles == (uint32_t)nblk && (kStep == kDirCursors || !dec_all_dirs(ws))) return;   // one tile each
     const DecWs W = dec_ws(ws, nblk);
     const int warp = threadIdx.x >> 5;
-    for (uint32_t gt = blockIdx.x * kDecWarps + warp; gt < tiles; gt += gridDim.x * kDecWarps) {
+    const uint32_t ways = kStep == kDirCursors ? 1u : dir_ways(tiles);   // (items of a tile)
+    for (uint32_t g = blockIdx.x * kDecWarps + warp; g < tiles * ways; g += gridDim.x * kDecWarps) {
+        const uint32_t gt = g / ways;
         const int b = find_block_warp(W.blk_tile, nblk, gt, (int)((uint64_t)gt * (uint32_t)nblk / tiles));
-        const uint32_t k = gt - W.blk_tile[b];
+        const uint32_t k = g - W.blk_tile[b] * ways;
         if (kStep == kDirShare) dir_share(b, k, comp, comp_off, nblk, ws, ws_bytes, status);
         else if (kStep == kDirCursors) dir_cursors(b, k, comp, comp_off, nblk, ws, ws_bytes, status);
         else dir_rebase(b, k, comp, comp_off, nblk, ws, ws_bytes, status);
@@ -2301,7 +2318,7 @@ __global__ void __launch_bounds__(kDecThreads, kTileCtas) decode_kernel(const ui
 //              from the plan's tables in shared memory
 //              (plans are in ticket order, as their look-back needs)
 //   ANS        8 units per item, one warp each
-//   shares     8 directory shares per item, one warp each
+//   shares     8 directory shares per item (`ways` to a tile), one warp each
 //   cursors    8 tile boundaries per item, one warp each
 //   tiles      one tile per item (cta_tile)
 // An item only waits (bounded) on items earlier in the queue: the ANS and
@@ -2381,20 +2398,23 @@ __device__ inline uint32_t batch_plans(const BatchQueue &q) { return q.wide ? ba
 // Items of each stage once all plans are done (header written by the last
 // plan; word 12 counts the blocks whose tiles are still to be decoded).
 struct BatchStages {
-    uint32_t ans, dir, tiles;   // ANS items; share items (as many cursor items); tile items
+    uint32_t ans, ways, shares, cursors, tiles;   // ANS items; shares of a tile, share items; cursor items; tile items
 };
 __device__ inline BatchStages batch_stages(const BatchQueue &q) {
     const uint32_t *hdr = reinterpret_cast<const uint32_t *>(q.ws);
     BatchStages s;
     const uint32_t left = *reinterpret_cast<const volatile uint32_t *>(&hdr[12]);
     s.ans = (hdr[2] + kAnsWarps - 1) / kAnsWarps;
-    s.dir = hdr[6] == (uint32_t)q.nblk ? 0u : (hdr[6] + kDecWarps - 1) / kDecWarps;   // (one tile each: no directory)
+    s.ways = dir_ways(hdr[6]);
+    const bool dir = hdr[6] != (uint32_t)q.nblk;   // (one tile each: no directory)
+    s.shares = dir ? (hdr[6] * s.ways + kDecWarps - 1) / kDecWarps : 0u;
+    s.cursors = dir ? (hdr[6] + kDecWarps - 1) / kDecWarps : 0u;
     s.tiles = left ? hdr[6] : 0u;
     return s;
 }
 __device__ inline uint32_t batch_items_total(const BatchQueue &q) {
     const BatchStages s = batch_stages(q);
-    return batch_items_blocks(q) + s.ans + 2 * s.dir + s.tiles;
+    return batch_items_blocks(q) + s.ans + s.shares + s.cursors + s.tiles;
 }
 
 // Block b's item: its plan and, when it needs nothing else, its decode.
@@ -2585,18 +2605,18 @@ __device__ __noinline__ int batch_item(const BatchQueue &q, uint32_t item, const
         return kItemDone;
     }
     it -= stg.ans;
-    if (it < 2 * stg.dir) {
-        // ---- directory shares, then cursors: one tile's per warp ----
-        const bool cursors = it >= stg.dir;
-        const uint32_t gt = (cursors ? it - stg.dir : it) * kDecWarps + warp;
+    if (it < stg.shares + stg.cursors) {
+        // ---- directory shares, then cursors: one per warp ----
+        const bool cursors = it >= stg.shares;
+        const uint32_t ways = cursors ? 1u : stg.ways, g = (cursors ? it - stg.shares : it) * kDecWarps + warp, gt = g / ways;
         if (gt < total_tiles) {
             const int b = find_block_warp(W.blk_tile, nblk, gt, (int)((uint64_t)gt * (uint32_t)nblk / total_tiles));
-            const uint32_t ntile = W.blk_ntile[b], k = gt - W.blk_tile[b];
+            const uint32_t ntile = W.blk_ntile[b], k = g - W.blk_tile[b] * ways;
             if (ntile > 1) {
                 int okw = 1;
                 if (lane == 0) {
                     const uint32_t nsegs = (b + 1 < nblk ? W.blk_seg[b + 1] : total_segs) - W.blk_seg[b];
-                    okw = cursors ? wait_geq(&W.dir_done[b], ntile, wait_bound(q))
+                    okw = cursors ? wait_geq(&W.dir_done[b], ntile * stg.ways, wait_bound(q))
                                   : wait_geq(&W.segs_done[b], nsegs, wait_bound(q));
                     if (!okw) q.status[b] = PIVCO_ERR_TIMEOUT;
                 }
@@ -2610,7 +2630,7 @@ __device__ __noinline__ int batch_item(const BatchQueue &q, uint32_t item, const
         __syncthreads();
         return kItemDone;
     }
-    it -= 2 * stg.dir;
+    it -= stg.shares + stg.cursors;
     if (it >= stg.tiles) return kItemNone;
     // ---- tile it: after its block's ANS segments and cursors (a block
     // decoded by its own item is skipped) ----
@@ -2623,7 +2643,7 @@ __device__ __noinline__ int batch_item(const BatchQueue &q, uint32_t item, const
             } else {
                 const uint32_t nsegs = (b + 1 < nblk ? W.blk_seg[b + 1] : total_segs) - W.blk_seg[b];
                 okw = wait_geq(&W.segs_done[b], nsegs, wait_bound(q));
-                if (okw && W.blk_ntile[b] > 1) okw = wait_geq(&W.dir_done[b], 2 * W.blk_ntile[b], wait_bound(q));
+                if (okw && W.blk_ntile[b] > 1) okw = wait_geq(&W.dir_done[b], (stg.ways + 1) * W.blk_ntile[b], wait_bound(q));
                 if (!okw) q.status[b] = PIVCO_ERR_TIMEOUT;
             }
             B.blk = b;
