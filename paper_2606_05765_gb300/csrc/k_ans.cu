@@ -145,18 +145,19 @@ cudaError_t launch_ans_decode(const uint8_t *bodies, const uint64_t *body_off, c
 //           the sb bytes of the workspace that mirror its place in the record:
 //           its word count and states at the start, its words at the end (they
 //           are emitted backwards, so they come out in the decoder's order).
-//           A segment that does not fit there is marked.
-//   place   one CTA per block: sizes, the choice per node, the rewrite.  A marked
-//           last segment (short ones have no room for their states) is coded
-//           here; a block with another marked one, or with no room for the
-//           mirror, by one warp, node after node.
+//           A segment that does not fit there is marked, with its word count.
+//   place   one CTA per block: sizes, the choice per node, the rewrite.  The
+//           marked segments of a node that is coded all the same, and last
+//           segments too short for a mirror, are coded here, a warp each; a
+//           block of many, or with no room for the mirror, by one warp, node
+//           after node.
 // What bounds it: the latency of a round's chain, 512 rounds a unit: the bytes
 // and table entries of 8 rounds are loaded before the chain needs them.  One
 // warp per block coded its nodes one after another: 236 us for 2048 bitmaps of
 // 16 KiB (one unit each), now 85 + 30 us; 445 us for 1024 blocks of many nodes,
 // now 57 + 31 us.
 // ---------------------------------------------------------------------------
-// One block by one warp (a segment of it did not fit its mirror).
+// One block by one warp (no room for its mirror, or too many marked segments).
 __device__ __noinline__ void ans_encode_block_serial(int b, const BlockLayout *__restrict__ layout, uint8_t *__restrict__ out,
                                                      const uint64_t *__restrict__ out_off,
                                                      uint64_t *__restrict__ rec_bytes, uint8_t *__restrict__ ws,
@@ -255,8 +256,9 @@ __device__ __noinline__ void ans_encode_block_serial(int b, const BlockLayout *_
 }
 
 
-constexpr uint32_t kAnsMirrorMin = 16;    // shorter segments have no room for their header: coded serially
-constexpr uint32_t kAnsMarked = 0xFFFFFFFFu;
+constexpr uint32_t kAnsMirrorMin = 16;    // shorter segments have no room for their header: coded by the place kernel
+constexpr uint32_t kAnsMarked = 0x80000000u;   // with the word count of a segment that does not fit its mirror
+constexpr uint32_t kAnsMarks = 64;        // marked segments of a block the place kernel codes itself
 
 struct AnsEncGroup {            // a segment of a unit
     uint32_t at, sb;            // its bytes in the record
@@ -432,7 +434,7 @@ __global__ void __launch_bounds__(32) ans_encode_units_kernel(const BlockLayout 
         else code(std::false_type{});
         // word count and states at the mirror's start (any byte)
         if (on) {
-            if (li == 0) st_le32(lo, nw <= cap ? nw : kAnsMarked);
+            if (li == 0) st_le32(lo, nw <= cap ? nw : kAnsMarked | nw);
             if (nw <= cap) st_le32(lo + 4 + 4 * li, x);
         }
     }
@@ -466,7 +468,8 @@ __global__ void __launch_bounds__(kAnsPlaceThreads, 8) ans_encode_place_kernel(c
     __shared__ uint32_t s_len[256];      // coded bytes of a node (0: kept raw)
     __shared__ uint32_t s_node[256];     // the selected nodes, in order
     __shared__ uint32_t s_n, s_nw, s_x[32];
-    __shared__ bool s_tail[256];         // the node's last segment is coded here
+    __shared__ bool s_tail[256];         // the node's last segment, without a mirror, is coded here
+    __shared__ uint32_t s_nmark, s_mark[kAnsMarks][3];   // marked segments of coded nodes: k, segment, words
     __shared__ AnsSm s_T[kAnsPlaceThreads / 32];
     extern __shared__ __align__(16) uint8_t sm[];
     uint16_t *stage = reinterpret_cast<uint16_t *>(sm + ((sizeof(AnsSm) + 15) & ~15));
@@ -485,23 +488,23 @@ __global__ void __launch_bounds__(kAnsPlaceThreads, 8) ans_encode_place_kernel(c
             if (sel) s_node[n + __popc(m & ((1u << lane) - 1u))] = v;
             n += __popc(m);
         }
-        if (lane == 0) s_n = n;
+        if (lane == 0) { s_n = n; s_nmark = 0; }
     }
     __syncthreads();
     const uint32_t nsel = s_n;
-    bool serial = out_off[b + 1] > ws_bytes;
+    bool serial = out_off[b + 1] > ws_bytes;   // (the same in every thread)
     // ---- sizes: a warp takes a node, its lanes the segments ----
     if (!serial)
         for (uint32_t k = warp; k < nsel; k += kAnsPlaceThreads / 32) {
             const uint32_t v = s_node[k], raw = (L.nv[v] + 7) / 8, S = ans_seg_count(raw), at = L.body_off[v];
             uint64_t sum = 0;
-            bool tail = false;
+            bool tail = false, marks = false;
             for (uint32_t s = lane; s < S; s += 32) {
                 const uint32_t sb = min(kAnsSeg, raw - s * kAnsSeg);
-                const uint32_t nw = sb >= kAnsMirrorMin ? ld_le32(mir + at + s * kAnsSeg) : kAnsMarked;
-                if (nw != kAnsMarked) sum += 4 + 4 * ans_seg_lanes(sb) + 2ull * nw;
-                else if (sb < kAnsSeg) tail = true;
-                else serial = true;
+                if (sb < kAnsMirrorMin) { tail = true; continue; }
+                const uint32_t nw = ld_le32(mir + at + s * kAnsSeg);
+                sum += 4 + 4 * ans_seg_lanes(sb) + 2ull * (nw & ~kAnsMarked);
+                if (nw & kAnsMarked) marks = true;
             }
             tail = __any_sync(0xffffffffu, tail);
 #pragma unroll
@@ -514,17 +517,32 @@ __global__ void __launch_bounds__(kAnsPlaceThreads, 8) ans_encode_place_kernel(c
                 __syncwarp();
                 const uint32_t nw = ans_encode_segment(rec + at + raw - sb, sb, s_T[warp], (mk & 0x80) ? 0xFF : 0, stage, 0u,
                                                        nullptr, 0u, x);
-                if (nw > kAnsStageWords) serial = true;
                 sum += 4 + 4 * ans_seg_lanes(sb) + 2ull * nw;
             }
+            if (marks && sum < raw)
+                for (uint32_t s = lane; s < S; s += 32) {
+                    if (min(kAnsSeg, raw - s * kAnsSeg) < kAnsMirrorMin) continue;
+                    const uint32_t nw = ld_le32(mir + at + s * kAnsSeg);
+                    if (!(nw & kAnsMarked)) continue;
+                    const uint32_t i = atomicAdd(&s_nmark, 1u);
+                    if (i < kAnsMarks) { s_mark[i][0] = k; s_mark[i][1] = s; s_mark[i][2] = nw & ~kAnsMarked; }
+                }
             if (lane == 0) { s_len[k] = sum < raw ? (uint32_t)sum : 0u; s_tail[k] = tail; }
         }
-    if (__syncthreads_or(serial)) {
+    __syncthreads();
+    const uint32_t nmark = s_nmark;
+    if (serial || nmark > kAnsMarks) {
         if (warp == 0) ans_encode_block_serial(b, layout, out, out_off, rec_bytes, ws, ws_bytes, A);
         return;
     }
+    // the marked segments' bytes into their mirrors, where the rewrite leaves them alone
+    for (uint32_t i = 0; i < nmark; i++) {
+        const uint32_t v = s_node[s_mark[i][0]], raw = (L.nv[v] + 7) / 8, o = s_mark[i][1] * kAnsSeg;
+        copy_words(ws + out_off[b] + L.body_off[v] + o, rec + L.body_off[v] + o, min(kAnsSeg, raw - o), t, kAnsPlaceThreads);
+    }
+    if (nmark) __syncthreads();
     // ---- rewrite the selected region in breadth-first order ----
-    // A node with its last segment marked, and one kept raw, reads the record:
+    // A node with a last segment without a mirror, and one kept raw, reads the record:
     // all the nodes up to it are in place before the next is begun.  The others
     // read the mirror, and end before the next node's raw copy: the warps take
     // their pieces in turn, and run ahead as far as no such node stands between.
@@ -554,12 +572,31 @@ __global__ void __launch_bounds__(kAnsPlaceThreads, 8) ans_encode_place_kernel(c
             for (uint32_t s = 0; s < S; s++) {
                 const uint32_t sb = min(kAnsSeg, raw - s * kAnsSeg), W = ans_seg_lanes(sb);
                 const uint8_t *lo = mir + at + s * kAnsSeg;
-                const bool marked = tail && s == S - 1;
-                const uint32_t nw = marked ? s_nw : ld_le32(lo);
+                const bool staged = tail && s == S - 1;
+                uint32_t mark = kAnsMarks;
+                for (uint32_t i = 0; i < nmark; i++)
+                    if (s_mark[i][0] == k && s_mark[i][1] == s) mark = i;
+                const uint32_t nw = mark < kAnsMarks ? s_mark[mark][2] : (staged ? s_nw : ld_le32(lo));
+                if (mark < kAnsMarks) {   // by one warp, its words straight to their place
+                    if (turn++ % kAnsPlaceWarps == (uint32_t)warp) {
+                        const uint32_t mk = L.sel[v];
+                        uint32_t x;
+                        __syncwarp();
+                        load_ans_table(s_T[warp], A, (mk & 0x7F) - 1, lane, 32, true);
+                        __syncwarp();
+                        ans_encode_segment(lo, sb, s_T[warp], (mk & 0x80) ? 0xFF : 0, stage, 0u, rec + p + 4 * W, nw, x);
+                        __syncwarp();
+                        ans_place_words(stage, 0u, nw, rec + p + 4 * W);
+                        if (lane < 4) rec[q + 4 * s + lane] = (uint8_t)(nw >> (8 * lane));
+                        if (lane < (int)W) st_le32(rec + p + 4 * lane, x);
+                    }
+                    p += 4 * W + 2 * nw;
+                    continue;
+                }
                 if (turn++ % kAnsPlaceWarps == (uint32_t)warp) {
                     if (lane < 4) rec[q + 4 * s + lane] = (uint8_t)(nw >> (8 * lane));
-                    if (lane < (int)W) st_le32(rec + p + 4 * lane, marked ? s_x[lane] : ld_le32(lo + 4 + 4 * lane));
-                    if (marked) {
+                    if (lane < (int)W) st_le32(rec + p + 4 * lane, staged ? s_x[lane] : ld_le32(lo + 4 + 4 * lane));
+                    if (staged) {
                         const uint16_t *wb = stage + kAnsStageWords - nw;
                         for (uint32_t i = lane; i < nw; i += 32) {
                             rec[p + 4 * W + 2 * i] = (uint8_t)wb[i];
@@ -567,7 +604,7 @@ __global__ void __launch_bounds__(kAnsPlaceThreads, 8) ans_encode_place_kernel(c
                         }
                     }
                 }
-                if (!marked) {   // 1 KiB at a time to a warp
+                if (!staged) {   // 1 KiB at a time to a warp
                     const uint8_t *wb = reinterpret_cast<const uint8_t *>((reinterpret_cast<uintptr_t>(lo) + sb) & ~(uintptr_t)1) - 2 * nw;
                     for (uint32_t i = 0; i < 2 * nw; i += 1024)
                         if (turn++ % kAnsPlaceWarps == (uint32_t)warp)
