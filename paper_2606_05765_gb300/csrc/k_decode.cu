@@ -54,6 +54,9 @@ __device__ inline uint32_t dec_dir_bits(const uint8_t *ws) { return reinterpret_
 __device__ inline bool dec_all_dirs(const uint8_t *ws) { return (reinterpret_cast<const uint32_t *>(ws)[7] >> 31) != 0; }
 
 __host__ __device__ inline uint32_t scratch_stride(uint32_t raw) { return ((raw + 15u) & ~15u) + 16u; }
+// scratch of a block's ANS-coded nodes at most (with the last one's 16 bytes of padding: bit addresses stay below
+// 2^31; a corrupt record's counts could ask for more than 2^32 bytes, and get a place over its neighbours')
+constexpr uint64_t kScratchMax = (1ull << 28) + 16;
 
 // The dynamic shared memory of every kernel here: the merge's selector table
 // (1 KiB), then what the item at hand needs.  The big steps are functions of
@@ -407,7 +410,10 @@ __device__ __noinline__ PlanRes plan_cta(const uint8_t *__restrict__ rec, uint64
     uint32_t scratch = 0, nsegs = 0;
     if (nsel) {
         const uint32_t rawb = (nv + 7) / 8;
-        Q.soff[t] = scan_cta(ans ? scratch_stride(rawb) : 0u, Q.wsum, scratch);
+        uint64_t tot;
+        Q.soff[t] = (uint32_t)scan_cta64(ans ? scratch_stride(rawb) : 0u, Q.wsum64[0], tot);
+        if (tot > kScratchMax) bad = true;
+        scratch = (uint32_t)tot;
         uint32_t full, lanes;
         scan_cta(ans ? ans_full_segs(rawb) : 0u, Q.wsum, full);
         scan_cta(ans ? ans_tail_lanes(rawb) : 0u, Q.wsum, lanes);
@@ -599,7 +605,7 @@ __device__ inline PlanRes plan_warp(const uint8_t *__restrict__ rec, uint64_t av
         nsel += __popc(__ballot_sync(0xffffffffu, v0 + lane < V && mark_listed(mks[min(v0 + lane, V - 1)])));
     const uint32_t alen_off = (kNvOff + 5 * V + 3) & ~3u, base1 = alen_off + 4 * nsel;
     if (base1 > rb) return R;
-    uint64_t raw_tot = 0, sel_tot = 0;
+    uint64_t raw_tot = 0, sel_tot = 0, scratch_tot = 0;
     uint32_t scratch = 0, full = 0, lanes = 0, ent = 0, np = 0;
     for (uint32_t v0 = 0; v0 < V; v0 += 32) {
         const uint32_t v = v0 + lane;
@@ -640,12 +646,13 @@ __device__ inline PlanRes plan_warp(const uint8_t *__restrict__ rec, uint64_t av
             const uint32_t st = ans ? scratch_stride((nv + 7) / 8) : 0u, si = warp_inclusive(st);
             if (listed) Q.src[v] = ans ? (8u * (scratch + si - st)) | 0x80000000u : (uint32_t)(sel_tot + inc - x);
             scratch += __shfl_sync(0xffffffffu, si, 31);
+            scratch_tot += 16ull * __reduce_add_sync(0xffffffffu, st / 16);   // (32 strides of 2^29 bytes at most: 2^30)
             full += __reduce_add_sync(0xffffffffu, ans ? ans_full_segs((nv + 7) / 8) : 0u);
             lanes += __reduce_add_sync(0xffffffffu, ans ? ans_tail_lanes((nv + 7) / 8) : 0u);
             sel_tot += __shfl_sync(0xffffffffu, inc, 31);
         }
     }
-    if (((base1 + raw_tot + sel_tot + 15) & ~15ull) != rb) bad = true;
+    if (((base1 + raw_tot + sel_tot + 15) & ~15ull) != rb || scratch_tot > kScratchMax) bad = true;
     __syncwarp();
     if (nsel)
         for (uint32_t v = lane; v < V; v += 32)

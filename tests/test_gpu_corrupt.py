@@ -57,3 +57,39 @@ def test_demand_past_the_body_is_refused(P, flat, batched):   # noqa: F811
         for b in range(len(blocks)):
             if st[b] == 0:
                 assert np.array_equal(out[int(ooff[b]):int(ooff[b + 1])], blocks[b]), b
+
+
+def test_scratch_of_a_corrupt_record(P):   # noqa: F811
+    """255 ANS-coded nodes whose counts ask for more than 2^32 bytes of scratch:
+    refused by the plan (by one CTA a record, and by warps), not given a place
+    as small as the sum's low 32 bits."""
+    import torch
+    V, nv = 255, 8 * 17_000_000
+    S = (nv // 8 + 16383) // 16384
+    tail = (nv // 8) % 16384
+    alen = 4 * S + 128 * (S - 1) + 4 * ((tail + 511) // 512)
+    hdr = np.zeros((144 + 5 * V + 3) // 4 * 4 + 4 * V, np.uint8)
+    size = (hdr.size + V * alen + 15) & ~15
+    hdr[0:8] = np.array([size, nv], np.uint32).view(np.uint8)
+    hdr[8], hdr[10] = V, 2
+    hdr[12:16] = np.frombuffer(b"PVC1", np.uint8)
+    hdr[16:144] = 0x88                              # 256 codes of 8 bits
+    hdr[144:144 + 4 * V] = np.full(V, nv, np.uint32).view(np.uint8)
+    hdr[144 + 4 * V:144 + 5 * V] = 30
+    hdr[-4 * V:] = np.full(V, alen, np.uint32).view(np.uint8)
+    comp = torch.zeros(size, dtype=torch.uint8, device="cuda")
+    comp[:hdr.size] = torch.from_numpy(hdr).cuda()
+    assert V * ((nv // 8 + 15) // 16 * 16 + 16) >> 32
+    # (sizing alone: the plan is all that runs)
+    for n in (1, 700):
+        # the same record, then records of constant blocks
+        one = np.zeros(16, np.uint8)
+        one[0:8] = np.array([16, 5], np.uint32).view(np.uint8)
+        one[10], one[11] = 1, 7
+        one[12:16] = hdr[12:16]
+        buf = torch.cat([comp, torch.from_numpy(np.tile(one, n - 1)).cuda()])
+        coff = np.concatenate([[0], size + 16 * np.arange(n)])
+        d = P.Decoder(n)
+        d.prepare(buf, off64(coff))
+        st = d.status.cpu().numpy()
+        assert st[0] == P.ERR_CORRUPT and not st[1:].any()
