@@ -816,7 +816,8 @@ __device__ __noinline__ void plan_item(int item, const uint8_t *__restrict__ com
         if (lane == 0) {
             const bool simple = ok && !to && R.ntile == 1 && R.nsegs == 0 && !all_dirs;
             __threadfence();
-            atomicExch(&W.plan_done[b], simple ? 3u : 1u);
+            // (4: the block's item has given up waiting for this plan, and will not come again)
+            if ((atomicOr(&W.plan_done[b], simple ? 3u : 1u) & 4u) && ok) status[b] = PIVCO_ERR_TIMEOUT;
         }
     }
 }
@@ -2562,9 +2563,13 @@ __device__ __noinline__ int batch_item(const BatchQueue &q, uint32_t item, const
         if (item < nplan + (uint32_t)nblk) {
             const int b = (int)(item - nplan);
             if (t == 0) {
-                const int okw = wait_geq(&W.plan_done[b], 1u, wait_bound(q));
-                if (!okw) q.status[b] = PIVCO_ERR_TIMEOUT;
-                B.ok = okw ? (int)*reinterpret_cast<volatile uint32_t *>(&W.plan_done[b]) : 0;
+                // a wait that runs out leaves its mark in the same word as the plan: the one that comes second sees
+                // the other's, so the block does not read OK when the plan is merely late
+                uint32_t pd = 0;
+                if (wait_geq(&W.plan_done[b], 1u, wait_bound(q))) pd = *reinterpret_cast<volatile uint32_t *>(&W.plan_done[b]);
+                else if ((pd = atomicOr(&W.plan_done[b], 4u)) != 0) __threadfence();
+                else q.status[b] = PIVCO_ERR_TIMEOUT;
+                B.ok = (int)pd;
             }
             __syncthreads();
             const int pd = B.ok;

@@ -499,7 +499,7 @@ cudaError_t launch_ans_decode(const uint8_t *bodies, const uint64_t *body_off, c
 struct DecWs {
     uint64_t *states_a, *states_b, *blk_scratch, *blk_dir;
     uint32_t *blk_seg, *blk_tile, *blk_T, *blk_ntile, *segs_done, *dir_done;
-    uint32_t *plan_done;   // 1 | 2 (one tile, no ANS, no directory) once the block's plan is complete
+    uint32_t *plan_done;   // 1 | 2 (one tile, no ANS, no directory) once the block's plan is complete; 4: its item gave up first
 };
 __host__ __device__ inline size_t decode_ws_fixed_bytes(int nblk) {
     const size_t f = 64 + 32ull * nblk + 28ull * nblk;
