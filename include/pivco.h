@@ -125,8 +125,9 @@ pivco_status pivco_build_layout(const uint32_t *hist, const uint8_t *lens, int32
                                 int32_t *status, void *stream);
 
 /* pivco_histogram_chunks, pivco_code_lengths and pivco_build_layout in one
- * launch (one CTA per block; the block's counts and lengths stay on chip
- * between the steps).  Writes exactly what the three calls write: hist,
+ * launch (one CTA per block, whose counts and lengths stay on chip between the
+ * steps; in the smallest batches large blocks are counted by a cluster of
+ * eight, through chunk_hist).  Writes exactly what the three calls write: hist,
  * chunk_hist, lens, layout, rec_bound and status (the layout step's). */
 pivco_status pivco_plan_blocks(const uint8_t *in, const uint64_t *blk_off, int32_t nblk,
                                const pivco_params *params, uint32_t *hist, uint32_t *chunk_hist,
@@ -170,10 +171,13 @@ pivco_status pivco_encode_blocks(const uint8_t *in, const uint64_t *blk_off, int
  * status: a block is either refused (status[b] = PIVCO_ERR_INVALID_ARG) or,
  * when the sums it used are right after all, encoded exactly; nothing is
  * written outside each block's record.  A block whose levels do not fit
- * the encoder's buffers, or one of 16384 symbols and more in a batch of few
- * blocks, is coded chunk by chunk by several CTAs (a work list of (block,
- * chunk) items, or shares of chunks); each chunk starts at the node cursors its
- * preceding chunks' histograms give.  Both encode calls keep that work list
+ * the encoder's buffers, or one of 16384 symbols and more in a batch so small
+ * that the chunks of all its blocks run at once, is coded chunk by chunk by
+ * several CTAs (a work list of (block, chunk) items, or shares of chunks); each
+ * chunk starts at the node cursors its preceding chunks' histograms give.  In
+ * batches of more blocks than SMs the chunks' kernel starts while the other
+ * blocks are still coded; its wait for the list's order is bounded (the list's
+ * blocks report PIVCO_ERR_TIMEOUT).  Both encode calls keep that work list
  * in scratch words at the end of the layout records, so one layout serves
  * one encode call at a time. */
 pivco_status pivco_histogram_chunks(const uint8_t *in, const uint64_t *blk_off, int32_t nblk,
@@ -378,7 +382,8 @@ uint64_t pivco_launch_count(void);
 /* Bound of the library's device-side waits (process-wide, host).  Every
  * wait a kernel makes on work of another CTA (the decoupled look-backs of
  * pivco_exclusive_scan and of the decode plan, the batched decode's and the
- * serving loop's waits on earlier queue items) gives up after `ns`
+ * serving loop's waits on earlier queue items, the encoder's wait for the order
+ * of its list of big blocks) gives up after `ns`
  * nanoseconds of device time.  The blocks concerned then report
  * PIVCO_ERR_TIMEOUT (pivco_exclusive_scan: its status_out) and the kernel
  * returns; no block whose work was abandoned reports PIVCO_OK.  Applies to

@@ -35,9 +35,9 @@ namespace pv {
 
 constexpr int kDecThreads = 256;
 constexpr int kDecWarps = kDecThreads / 32;
-constexpr int kLvlFit = 24576;               // the plan's measure of a level buffer: tiles keep their levels below
-                                             // it by 20 %
+constexpr int kLvlFit = 24576;               // the plan's measure of a level (plan_tiles)
 constexpr int kLvlBuf = 23360;               // one level buffer of a tile (bytes; what is left of the shared memory)
+static_assert(4 * (kLvlFit - 4 * 128 - 32) / 5 + 15 * 128 <= kLvlBuf, "a tile of even statistics fits");
 constexpr int kWSlack = 80;                  // over-read room of the byte windows (64 symbols and 11 bytes)
 constexpr int kTileCtas = 4;                 // tile CTAs per SM the kernels are built for
 constexpr uint32_t kNtabHdr = 32;            // node table header (see plan_block)
@@ -214,8 +214,11 @@ __device__ inline bool plan_children(const PlanTree &P, const uint8_t *sorted, u
 }
 
 // Root symbols per tile and tiles of a block of n symbols (one warp; lvl[d]:
-// symbols of level d): every level of a tile must fit one level buffer (with
-// 4-byte rounding per node), with 20 % headroom.
+// symbols of level d): a tile's average share of every level is at most 4/5 of
+// kLvlFit - 32 bytes, less 4 bytes a node.  With the spans' 15 bytes of rounding
+// a node at most, that leaves 16 % of the level buffer free for a level of few
+// nodes, 10 % for one of 128; a tile that needs more (the block's statistics
+// drift) is decoded in chunks.
 __device__ inline void plan_tiles(const PlanTree &P, const uint32_t *lvl, uint32_t n, uint32_t tile_max, uint32_t &T,
                                   uint32_t &ntile) {
     const int lane = threadIdx.x & 31;

@@ -60,10 +60,10 @@ struct __align__(16) EncSmem {
     uint32_t lut[256];                      // byte selectors that bring the symbols of a bitmap byte's zeros to the
                                             // front (first four in the low half)
     uint32_t pmask[8];                      // symbols that have a code
-    uint32_t bad, lvl_max;                  // symbols of the largest level below the root (a part that did not fit)
+    uint32_t bad;                           // the part's symbols do not match its counts
     uint8_t first[17];
     uint8_t maxd;
-    uint8_t pad[14];
+    uint8_t pad[2];
 };
 static_assert(kEncCtasPerSm * (sizeof(EncSmem) + 64 + 1024) <= 228 * 1024, "encoder CTAs per SM");
 static_assert(offsetof(BlockLayout, ci) <= sizeof(EncSmem::buf[1]) && offsetof(BlockLayout, ci) % 16 == 0,
@@ -86,27 +86,6 @@ __device__ inline uint32_t warp_scan_loop(int n, F f, G out) {
         carry += __shfl_sync(0xffffffffu, inc, 31);
     }
     return carry;
-}
-
-// 32 input bytes at p (any alignment; bytes at or past `end` read as 0)
-__device__ inline void ldg32(const uint8_t *p, const uint8_t *end, uint32_t (&x)[8]) {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-    if (!(a & 15) && p + 32 <= end) {
-        const uint4 u0 = __ldg(reinterpret_cast<const uint4 *>(p)), u1 = __ldg(reinterpret_cast<const uint4 *>(p) + 1);
-        x[0] = u0.x; x[1] = u0.y; x[2] = u0.z; x[3] = u0.w;
-        x[4] = u1.x; x[5] = u1.y; x[6] = u1.z; x[7] = u1.w;
-        return;
-    }
-    const uint32_t *w = reinterpret_cast<const uint32_t *>(a & ~uintptr_t(3));
-    const uint32_t sh = (uint32_t)(a & 3) * 8;
-    const uint8_t *wend = reinterpret_cast<const uint8_t *>(w);
-    uint32_t prev = wend < end ? __ldg(w) : 0u;
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-        const uint32_t nx = (wend + 4 * (j + 1) < end) ? __ldg(w + j + 1) : 0u;
-        x[j] = sh ? __funnelshift_r(prev, nx, sh) : prev;
-        prev = nx;
-    }
 }
 
 // Node symbol counts of a histogram h by prefix sums in canonical order: the
@@ -830,10 +809,10 @@ __device__ inline void encode_item(int b, uint32_t cA, uint32_t share, uint32_t 
     __syncthreads();
 }
 
-// The big blocks of a chunked encode (their levels do not fit the buffers):
-// checked, their bodies zeroed and their status set OK, and listed; then
-// every chunk of theirs is an item of the encode kernel's work list.  One
-// CTA per block.
+// The big blocks of a chunked encode (BlockLayout::big): checked, their bodies
+// zeroed and their status set OK, and listed; then every chunk of theirs, or
+// every share of one, is an item of the chunk kernel's work list.  gridDim.y
+// CTAs zero a block.
 __global__ void __launch_bounds__(kEncThreads) encode_reset_kernel(const uint64_t *__restrict__ blk_off,
                                                                    BlockLayout *__restrict__ layout,
                                                                    uint8_t *__restrict__ out,
