@@ -155,7 +155,9 @@ cudaError_t launch_ans_decode(const uint8_t *bodies, const uint64_t *body_off, c
 // and table entries of 8 rounds are loaded before the chain needs them.  One
 // warp per block coded its nodes one after another: 236 us for 2048 bitmaps of
 // 16 KiB (one unit each), now 85 + 30 us; 445 us for 1024 blocks of many nodes,
-// now 57 + 31 us.
+// now 57 + 31 us.  Where half of each block is noise, whole encode calls: 1 MiB
+// 1909 us before, 2171 with every marked segment left to the one warp, 482 now;
+// 64 blocks of 256 KiB 536, 609 and 328.
 // ---------------------------------------------------------------------------
 // One block by one warp (no room for its mirror, or too many marked segments).
 __device__ __noinline__ void ans_encode_block_serial(int b, const BlockLayout *__restrict__ layout, uint8_t *__restrict__ out,

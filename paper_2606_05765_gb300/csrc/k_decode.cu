@@ -138,7 +138,7 @@ static_assert(kStage >= kNvOff + 5 * 255 + 3 + 4 * 255 && kStage % 16 == 0, "the
 // What bounds it: latency, a chain of about twelve short steps per record.
 // A whole CTA takes a record (thread t is node t and symbol t) so that a
 // step is one instruction sequence and a barrier instead of a warp's loop
-// over 256 items: one record alone is planned in 9 us against 25 us by one
+// over 256 items: one record alone is planned in 8 us against 25 us by one
 // warp.
 // ---------------------------------------------------------------------------
 struct PlanTree {
@@ -2042,12 +2042,13 @@ __device__ __noinline__ void tile_close(int how, int nblk, const uint8_t *__rest
 //             shares between the node's start and the entry
 // What bounds them: the latency of dependent reads (a share's windows one
 // after another, a boundary's levels one after another).  One CTA per block
-// took 242 us for a block of 2^20 symbols alone; shares and cursors take 44 +
-// 29 us.
+// took 242 us for a block of 2^20 symbols alone; as many shares as tiles at
+// most, and their cursors, 43 + 29 us; eight times as many 30 + 33.
 // ---------------------------------------------------------------------------
 constexpr uint32_t kDirShares = 128;   // shares of a block at most
 constexpr uint32_t kDirShareMin = 10;  // log2 of the fewest entries of a share (but for the block's last) ...
-constexpr uint32_t kDirShareFew = 7;   // ... in batches of few tiles: one step of dir_share_count
+constexpr uint32_t kDirShareFew = 7;   // ... in batches of few tiles: one step of dir_share_count (300 blocks of two
+                                       // tiles and 860 entries: 36 us by one share each, 18 by seven)
 constexpr uint32_t kDirTarget = 4864;  // about as many shares as warps of the pass run at once (four CTAs an SM)
 constexpr uint32_t kDirWays = 8;
 
@@ -2392,9 +2393,10 @@ __device__ inline uint64_t wait_bound(const BatchQueue &q) { return reinterpret_
 // Plans by warps, then the blocks' own items (a wide batch): for more blocks than
 // the launch has CTAs, where the plans' instructions count (4096 blocks of
 // 64 KiB: 150 us of CTA plans, 50 us of warp plans; the line stands where the
-// second wave begins: 862 blocks decode in 166 us by warp plans, 185 by CTA
-// plans); else one item plans and decodes a block, its decode starting 7 us
-// after the item (a warp plan takes 25 us).  Decided once per batch: the items of
+// second wave begins: 862 blocks of 1 to 16 KB decode in 73 to 96 us by warp
+// plans, 78 to 99 by CTA plans, 640 in 68 to 87 and 64 to 84); else one item plans
+// and decodes a block, its decode starting 6 us after the item (a warp plan takes
+// 25 us).  Decided once per batch: the items of
 // a served request are taken by several launches, which need not have the same
 // number of CTAs (the tuning may change between them), so its form goes with
 // the request.

@@ -3,9 +3,9 @@
 // One CTA encodes one block, top-down, level by level; its warps share two
 // level buffers.  A block whose levels fit them is coded in one part (the
 // planning pass's chunk histograms give every node's symbol count); a big
-// block is coded in parts of a length the plan has chosen, by several CTAs
-// (one planning chunk, or a share of one, each), a part's counts taken from
-// the input.  A node's bitmap holds, in block order, the code bit of every
+// block (one whose levels do not fit, or one of a small batch) is coded in
+// parts of a length the plan has chosen, by several CTAs (one planning chunk,
+// or a share of one, each), a part's counts taken from the input.  A node's bitmap holds, in block order, the code bit of every
 // symbol passing through it, so a part's bits of node v start at the symbols
 // under v in the parts before it: the cursors advance by each part's counts.
 //
