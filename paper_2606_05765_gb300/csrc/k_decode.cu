@@ -57,6 +57,9 @@ __host__ __device__ inline uint32_t scratch_stride(uint32_t raw) { return ((raw 
 // scratch of a block's ANS-coded nodes at most (with the last one's 16 bytes of padding: bit addresses stay below
 // 2^31; a corrupt record's counts could ask for more than 2^32 bytes, and get a place over its neighbours')
 constexpr uint64_t kScratchMax = (1ull << 28) + 16;
+// and a node's bits in the record end below that too (bitmaps that are not ANS-coded; nothing later could tell
+// their addresses from the scratch's)
+__device__ inline bool body_far(uint64_t off, uint32_t nv, uint32_t fd) { return 8 * off + (uint64_t)nv * (fd ? fd : 1u) >= 1ull << 31; }
 
 // The dynamic shared memory of every kernel here: the merge's selector table
 // (1 KiB), then what the item at hand needs.  The big steps are functions of
@@ -408,7 +411,7 @@ __device__ __noinline__ PlanRes plan_cta(const uint8_t *__restrict__ rec, uint64
         const uint64_t so = scan_cta64(listed ? al : 0u, Q.wsum64[1], sel_tot);
         if (listed) off = base1 + raw_tot + so;
     }
-    if (((base1 + raw_tot + sel_tot + 15) & ~15ull) != rb) bad = true;
+    if (((base1 + raw_tot + sel_tot + 15) & ~15ull) != rb || (node && !ans && body_far(off, nv, fd))) bad = true;
     Q.body_off[t] = (uint32_t)off;
     uint32_t scratch = 0, nsegs = 0;
     if (nsel) {
@@ -635,7 +638,10 @@ __device__ inline PlanRes plan_warp(const uint8_t *__restrict__ rec, uint64_t av
             const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
             if (lane >= o) inc += y;
         }
-        if (node && !listed) Q.src[v] = 8u * (uint32_t)(base1 + raw_tot + inc - x);
+        if (node && !listed) {
+            Q.src[v] = 8u * (uint32_t)(base1 + raw_tot + inc - x);
+            if (body_far(base1 + raw_tot + inc - x, nv, fd)) bad = true;
+        }
         raw_tot += __shfl_sync(0xffffffffu, inc, 31);
         if (lm) {
             x = listed ? al : 0u;
@@ -659,7 +665,10 @@ __device__ inline PlanRes plan_warp(const uint8_t *__restrict__ rec, uint64_t av
     __syncwarp();
     if (nsel)
         for (uint32_t v = lane; v < V; v += 32)
-            if (mks[v] == kMarkRawSel) Q.src[v] = 8u * (uint32_t)(base1 + raw_tot + Q.src[v]);
+            if (mks[v] == kMarkRawSel) {
+                if (body_far(base1 + raw_tot + Q.src[v], nvs[v], 0u)) bad = true;
+                Q.src[v] = 8u * (uint32_t)(base1 + raw_tot + Q.src[v]);
+            }
     // ---- symbols: their number within their length (rounds of 32), the tree, their order ----
     uint32_t rank[8];
 #pragma unroll
