@@ -650,6 +650,14 @@ __device__ inline void build_layout_block(int b, const uint32_t *h, const uint8_
                     c_raw += __shfl_sync(0xffffffffu, ir, 31);
                     c_sel += __shfl_sync(0xffffffffu, is, 31);
                 }
+                // the encoder's bit addresses are 32-bit words (blocks of up to 2^28 symbols stay below that with 15 bits each)
+                if (n > (1u << 28)) {
+                    uint64_t tot = 0;
+                    for (int v = lane; v < V; v += 32) tot += ((uint64_t)L.nv[v] * max(1u, (uint32_t)L.fd[v]) + 7) / 8;
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+                    if (off0 + tot > (1u << 29) - 16) st = PIVCO_ERR_INVALID_ARG;
+                }
                 if (lane == 0) {
                     L.body0 = off0;
                     L.n_sel = (uint8_t)nsel;

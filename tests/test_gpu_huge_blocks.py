@@ -2,7 +2,8 @@
 
 Bitmaps that end within the first 2^28 bytes of a record decode; a record with
 any later is refused by every decode call and by random access (whose walk
-reads them without a limit of its own)."""
+reads them without a limit of its own), and a block whose record would pass
+2^29 bytes is refused by the encoder's plan."""
 import numpy as np
 import pytest
 
@@ -40,3 +41,10 @@ def test_largest_record(P, n, want, batched):   # noqa: F811
     assert (qst == (P.ERR_CORRUPT if want else 0)).all()
     if not want:
         assert torch.equal(sym, data[pos.to(torch.int64)])
+
+
+def test_too_large_for_the_encoder(P):   # noqa: F811
+    n = (1 << 29) + 4096
+    e = P.Encoder(1)
+    e.plan(uniform(n), off64([0, n]))
+    assert int(e.status.cpu()[0]) == P.ERR_INVALID_ARG
