@@ -58,8 +58,8 @@ __host__ __device__ inline uint32_t scratch_stride(uint32_t raw) { return ((raw 
 // 2^31; a corrupt record's counts could ask for more than 2^32 bytes, and get a place over its neighbours')
 constexpr uint64_t kScratchMax = (1ull << 28) + 16;
 // and a node's bits in the record end below that too (bitmaps that are not ANS-coded; nothing later could tell
-// their addresses from the scratch's)
-__device__ inline bool body_far(uint64_t off, uint32_t nv, uint32_t fd) { return 8 * off + (uint64_t)nv * (fd ? fd : 1u) >= 1ull << 31; }
+// their addresses from the scratch's); only in a record of kRecFar bytes can they not
+constexpr uint32_t kRecFar = 1u << 28;
 
 // The dynamic shared memory of every kernel here: the merge's selector table
 // (1 KiB), then what the item at hand needs.  The big steps are functions of
@@ -329,6 +329,25 @@ __device__ inline uint64_t scan_cta64(uint64_t x, uint64_t *wsum, uint64_t &tota
     return base + inc - x;
 }
 
+// Whether a bitmap of a record of kRecFar bytes or more (staged at g) ends past
+// the bit addresses (every thread the same; out of the way of the others).
+__device__ __noinline__ bool plan_far(const uint8_t *g, uint32_t V, uint32_t nsel) {
+    const uint8_t *mks = g + kNvOff + 4 * V;
+    const uint32_t alen_off = (kNvOff + 5 * V + 3) & ~3u;
+    uint64_t off = alen_off + 4 * nsel;
+    bool far = false;
+    uint32_t k = 0;
+    for (int pass = 0; pass < 2; pass++)   // the raw and flat nodes' bodies, then the listed ones'
+        for (uint32_t v = 0; v < V; v++) {
+            const uint32_t mk = mks[v];
+            if (mark_listed(mk) != (pass == 1)) continue;
+            const uint64_t bits = (uint64_t)ld_le32(g + kNvOff + 4 * v) * max(1u, (uint32_t)mark_flat_d(mk));
+            if (!mark_ans(mk) && 8 * off + bits >= 1ull << 31) far = true;
+            off += pass ? ld_le32(g + alen_off + 4 * k++) : (bits + 7) / 8;
+        }
+    return far;
+}
+
 // Parses record b, checks its layout and builds its node table in Q (the
 // whole CTA, kDecThreads threads; nothing global is written).
 __device__ __noinline__ PlanRes plan_cta(const uint8_t *__restrict__ rec, uint64_t avail, uint32_t dir_bits,
@@ -411,7 +430,8 @@ __device__ __noinline__ PlanRes plan_cta(const uint8_t *__restrict__ rec, uint64
         const uint64_t so = scan_cta64(listed ? al : 0u, Q.wsum64[1], sel_tot);
         if (listed) off = base1 + raw_tot + so;
     }
-    if (((base1 + raw_tot + sel_tot + 15) & ~15ull) != rb || (node && !ans && body_far(off, nv, fd))) bad = true;
+    if (((base1 + raw_tot + sel_tot + 15) & ~15ull) != rb) bad = true;
+    if (rb >= kRecFar && plan_far(g, V, nsel)) bad = true;
     Q.body_off[t] = (uint32_t)off;
     uint32_t scratch = 0, nsegs = 0;
     if (nsel) {
@@ -638,10 +658,7 @@ __device__ inline PlanRes plan_warp(const uint8_t *__restrict__ rec, uint64_t av
             const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
             if (lane >= o) inc += y;
         }
-        if (node && !listed) {
-            Q.src[v] = 8u * (uint32_t)(base1 + raw_tot + inc - x);
-            if (body_far(base1 + raw_tot + inc - x, nv, fd)) bad = true;
-        }
+        if (node && !listed) Q.src[v] = 8u * (uint32_t)(base1 + raw_tot + inc - x);
         raw_tot += __shfl_sync(0xffffffffu, inc, 31);
         if (lm) {
             x = listed ? al : 0u;
@@ -665,10 +682,8 @@ __device__ inline PlanRes plan_warp(const uint8_t *__restrict__ rec, uint64_t av
     __syncwarp();
     if (nsel)
         for (uint32_t v = lane; v < V; v += 32)
-            if (mks[v] == kMarkRawSel) {
-                if (body_far(base1 + raw_tot + Q.src[v], nvs[v], 0u)) bad = true;
-                Q.src[v] = 8u * (uint32_t)(base1 + raw_tot + Q.src[v]);
-            }
+            if (mks[v] == kMarkRawSel) Q.src[v] = 8u * (uint32_t)(base1 + raw_tot + Q.src[v]);
+    if (rb >= kRecFar && plan_far(g, V, nsel)) bad = true;
     // ---- symbols: their number within their length (rounds of 32), the tree, their order ----
     uint32_t rank[8];
 #pragma unroll
